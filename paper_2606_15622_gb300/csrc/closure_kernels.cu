@@ -1,17 +1,18 @@
 // closure_kernels.cu -- moment gather and 9x9 assembly + pivoted solve
 // (paper Sec. 3.6-3.7) for sm_103a.
 //
-// Kernel 1 (gather): a group of G lanes per cell, static round-robin over the
-// cells.  Each group makes two passes over its cell's particles (contiguous,
-// coalesced loads of the SoA arrays):
+// Kernel 1 (gather, FP32 moments of arrays that gather_tile.cu does not take;
+// FP64 moments: gather_fp64.cu): a group of G lanes per cell, static
+// round-robin over the cells.  Each group makes two passes over its cell's
+// particles (contiguous, coalesced loads of the SoA arrays):
 //   pass A  mean offset m and spread from the first particle v0;
 //   pass B  the 25 central sums (u_ij, u_ijk, |c|^2 c_i c_j, |c|^4 c_i) and
 //           <|c|^6> (which the velocity update's <N.N> needs).
-// FP32 mode centres on v0 + m and scales by a power of two s ~ 1/sqrt(theta)
+// It centres on v0 + m and scales by a power of two s ~ 1/sqrt(theta)
 // (exact scaling), accumulates short blocks in FP32 and folds the blocks with
-// two-sum; the group reduction is a compensated reduce-scatter.  FP64 mode
-// accumulates plain FP64 sums about the exact mean.  The second pass re-reads
-// the cell from L1/L2, so DRAM traffic stays one read of the velocities.
+// two-sum; the group reduction is a compensated reduce-scatter.  The second
+// pass re-reads the cell from L1/L2, so DRAM traffic stays one read of the
+// velocities.
 //
 // Kernel 2 (solve): one THREAD per cell.  GB300's FP64 pipe issues one warp
 // instruction every ~16 cycles per SM whatever the active mask, so idle lanes
@@ -43,21 +44,6 @@ __device__ __forceinline__ void accumulate26(float (&t)[kNSum], float wx, float 
   const float r4 = r2 * r2;
   t[22] = fmaf(r4, wx, t[22]); t[23] = fmaf(r4, wy, t[23]); t[24] = fmaf(r4, wz, t[24]);
   t[25] = fmaf(r4, r2, t[25]);
-}
-
-__device__ __forceinline__ void accumulate26d(double (&t)[32], double cx, double cy, double cz) {
-  const double xx = cx * cx, xy = cx * cy, xz = cx * cz, yy = cy * cy, yz = cy * cz, zz = cz * cz;
-  t[0] += xx; t[1] += xy; t[2] += xz; t[3] += yy; t[4] += yz; t[5] += zz;
-  t[6] = fma(xx, cx, t[6]);  t[7] = fma(xx, cy, t[7]);   t[8] = fma(xx, cz, t[8]);
-  t[9] = fma(xy, cy, t[9]);  t[10] = fma(xy, cz, t[10]); t[11] = fma(xz, cz, t[11]);
-  t[12] = fma(yy, cy, t[12]); t[13] = fma(yy, cz, t[13]); t[14] = fma(yz, cz, t[14]);
-  t[15] = fma(zz, cz, t[15]);
-  const double r2 = xx + yy + zz;
-  t[16] = fma(r2, xx, t[16]); t[17] = fma(r2, xy, t[17]); t[18] = fma(r2, xz, t[18]);
-  t[19] = fma(r2, yy, t[19]); t[20] = fma(r2, yz, t[20]); t[21] = fma(r2, zz, t[21]);
-  const double r4 = r2 * r2;
-  t[22] = fma(r4, cx, t[22]); t[23] = fma(r4, cy, t[23]); t[24] = fma(r4, cz, t[24]);
-  t[25] = fma(r4, r2, t[25]);
 }
 
 template <typename VT>
@@ -206,59 +192,6 @@ __global__ void __launch_bounds__(256) gather_fp32_kernel(const VT *__restrict__
   }
 }
 
-template <typename VT, int G>
-__global__ void __launch_bounds__(256) gather_fp64_kernel(const VT *__restrict__ v, int64_t np,
-                                                          const int64_t *__restrict__ off, int64_t n_cells,
-                                                          double *__restrict__ mom, double *__restrict__ m6) {
-  constexpr int GPW = 32 / G;
-  constexpr int K = 32 / G;
-  const int lane = threadIdx.x & 31;
-  const int lg = lane & (G - 1);
-  const int g = lane / G;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const VT *vx = v, *vy = v + np, *vz = v + 2 * np;
-
-  for (int64_t base = warp * GPW; base < n_cells; base += nwarps * GPW) {
-    const int64_t c = base + g;
-    const bool valid = c < n_cells;
-    int64_t a = 0, e = 0;
-    if (valid) {
-      a = off[c];
-      e = off[c + 1];
-    }
-    const int n = (int)(e - a);
-    const int itmax = __reduce_max_sync(0xffffffffu, (n + G - 1) / G);
-    double sx = 0.0, sy = 0.0, sz = 0.0;
-    for (int it = 0; it < itmax; ++it) {
-      const int64_t p = a + (int64_t)it * G + lg;
-      if (p < e) {
-        sx += (double)ldg_v(vx + p);
-        sy += (double)ldg_v(vy + p);
-        sz += (double)ldg_v(vz + p);
-      }
-    }
-    sx = group_allreduce<G>(sx);
-    sy = group_allreduce<G>(sy);
-    sz = group_allreduce<G>(sz);
-    const double inv_nd = n > 0 ? 1.0 / (double)n : 0.0;
-    const double Ux = sx * inv_nd, Uy = sy * inv_nd, Uz = sz * inv_nd;
-    double t[32];
-#pragma unroll
-    for (int q = 0; q < 32; ++q) t[q] = 0.0;
-    for (int it = 0; it < itmax; ++it) {
-      const int64_t p = a + (int64_t)it * G + lg;
-      if (p < e)
-        accumulate26d(t, (double)ldg_v(vx + p) - Ux, (double)ldg_v(vy + p) - Uy, (double)ldg_v(vz + p) - Uz);
-    }
-    group_reduce_scatter<G>(t, lane);
-    double val[K];
-#pragma unroll
-    for (int j = 0; j < K; ++j) val[j] = t[j] * inv_nd;
-    store_moments<G>(val, valid, lane, c, n, Ux, Uy, Uz, mom, m6);
-  }
-}
-
 // ---------------------------------------------------------------------------
 // assembly + solve (closure_math.cuh)
 // ---------------------------------------------------------------------------
@@ -300,40 +233,33 @@ static int sm_count() {
 }
 
 template <int G>
-static void launch_gather_t(const void *v, int v_dtype, int64_t np, const int64_t *off, int64_t n_cells, int prec,
-                            double *mom, double *m6, cudaStream_t st) {
+static void launch_gather_fp32(const void *v, int v_dtype, int64_t np, const int64_t *off, int64_t n_cells,
+                               double *mom, double *m6, cudaStream_t st) {
   const int threads = 256;
   const int64_t groups_per_block = (threads / 32) * (32 / G);
   int64_t blocks = (n_cells + groups_per_block - 1) / groups_per_block;
   const int64_t cap = (int64_t)sm_count() * 8;
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
-  if (prec == FP_PREC_FP32_MOMENTS) {
-    if (v_dtype == FP_V_F32)
-      gather_fp32_kernel<float, G><<<(unsigned)blocks, threads, 0, st>>>((const float *)v, np, off, n_cells, mom, m6);
-    else
-      gather_fp32_kernel<double, G><<<(unsigned)blocks, threads, 0, st>>>((const double *)v, np, off, n_cells, mom,
-                                                                          m6);
-  } else {
-    if (v_dtype == FP_V_F32)
-      gather_fp64_kernel<float, G><<<(unsigned)blocks, threads, 0, st>>>((const float *)v, np, off, n_cells, mom, m6);
-    else
-      gather_fp64_kernel<double, G><<<(unsigned)blocks, threads, 0, st>>>((const double *)v, np, off, n_cells, mom,
-                                                                          m6);
-  }
+  if (v_dtype == FP_V_F32)
+    gather_fp32_kernel<float, G><<<(unsigned)blocks, threads, 0, st>>>((const float *)v, np, off, n_cells, mom, m6);
+  else
+    gather_fp32_kernel<double, G><<<(unsigned)blocks, threads, 0, st>>>((const double *)v, np, off, n_cells, mom, m6);
 }
 
 bool launch_gather_tile(const float *v, int64_t np, const int64_t *off, int64_t n_cells, double *mom, double *m6,
                         cudaStream_t st, int sm_count);
+void launch_gather_fp64(const void *v, int v_dtype, int64_t np, const int64_t *off, int64_t n_cells, double *mom,
+                        double *m6, cudaStream_t st, int sm_count);
 
 void launch_gather(const void *v, int v_dtype, int64_t np, const int64_t *off, int64_t n_cells, int prec,
                    double *mom, double *m6, cudaStream_t st) {
   // FP32 moments of FP32 velocities: shared-memory staged tiles (16-byte
-  // aligned velocity arrays); every other combination: direct loads.
-  if (prec == FP_PREC_FP32_MOMENTS && v_dtype == FP_V_F32 &&
-      launch_gather_tile((const float *)v, np, off, n_cells, mom, m6, st, sm_count()))
-    return;
-  launch_gather_t<8>(v, v_dtype, np, off, n_cells, prec, mom, m6, st);
+  // aligned velocity arrays); FP32 moments of other arrays: direct loads.
+  if (prec != FP_PREC_FP32_MOMENTS)
+    launch_gather_fp64(v, v_dtype, np, off, n_cells, mom, m6, st, sm_count());
+  else if (v_dtype != FP_V_F32 || !launch_gather_tile((const float *)v, np, off, n_cells, mom, m6, st, sm_count()))
+    launch_gather_fp32<8>(v, v_dtype, np, off, n_cells, mom, m6, st);
 }
 
 void launch_solve(const double *mom, const double *tau, int64_t n_cells, const fp_params &p, int prec,

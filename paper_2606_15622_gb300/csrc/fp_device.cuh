@@ -108,25 +108,9 @@ __device__ __forceinline__ T group_allreduce(T x) {
 }
 
 // Reduce-scatter of 32 slots over groups of G lanes: on return lane l of the
-// group holds, in v[0 .. 32/G), the group sums of slots [l*32/G, (l+1)*32/G).
-template <int G, typename T>
-__device__ __forceinline__ void group_reduce_scatter(T (&v)[32], int lane) {
-#pragma unroll
-  for (int lvl = 0; (G >> (lvl + 1)) >= 1; ++lvl) {
-    const int o = G >> (lvl + 1);
-    const int half = 16 >> lvl;
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int j = 0; j < half; ++j) {
-      T send = up ? v[j] : v[j + half];
-      T keep = up ? v[j + half] : v[j];
-      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-}
-
-// The same with (hi, lo) compensated pairs: hi sums by two-sum, errors and
-// lo parts accumulated in lo.
+// group holds, in hi / lo[0 .. 32/G), the group sums of slots [l*32/G,
+// (l+1)*32/G), as compensated pairs: hi sums by two-sum, errors and lo parts
+// accumulated in lo.
 template <int G>
 __device__ __forceinline__ void group_reduce_scatter2(float (&hi)[32], float (&lo)[32], int lane) {
 #pragma unroll

@@ -69,18 +69,19 @@ __device__ __forceinline__ void store_comp<double>(double *p, int cls, const dou
     p[0] = x[0], p[1] = x[1], p[2] = x[2], p[3] = x[3];
 }
 
-// The first cell c in [0, n] with off[c] >= t (off nondecreasing, off[n] >=
-// t), found by the 16 lanes of the calling half warp together: each round
-// probes 16 evenly spaced offsets and keeps the interval where the answer
-// lies, so 2^17 cells take five dependent loads.
-__device__ __forceinline__ int64_t lower_bound16(const int64_t *__restrict__ off, int64_t n, int64_t t, int lane) {
+// The first cell c in [0, n] with at(c) >= t (at nondecreasing, at(n) >= t),
+// found by the 16 lanes of the calling half warp together: each round probes
+// 16 evenly spaced cells and keeps the interval where the answer lies, so
+// 2^17 cells take five dependent loads.
+template <class At>
+__device__ __forceinline__ int64_t lower_bound16_by(At at, int64_t n, int64_t t, int lane) {
   const int h = lane & 15;
   const unsigned hmask = 0xffffu << (lane & 16);
   int64_t lo = 0, hi = n;  // the answer lies in [lo, hi]
   while (hi - lo > 15) {
     const int64_t step = (hi - lo + 15) / 16;
     const int64_t c = min(lo + step * h, hi);
-    const unsigned b = (__ballot_sync(hmask, off[c] >= t) >> (lane & 16)) & 0xffffu;
+    const unsigned b = (__ballot_sync(hmask, at(c) >= t) >> (lane & 16)) & 0xffffu;
     if (b == 0) {
       lo = min(lo + step * 15, hi) + 1;
     } else {
@@ -94,8 +95,13 @@ __device__ __forceinline__ int64_t lower_bound16(const int64_t *__restrict__ off
     }
   }
   const int64_t c = min(lo + h, hi);
-  const unsigned b = (__ballot_sync(hmask, off[c] >= t) >> (lane & 16)) & 0xffffu;
+  const unsigned b = (__ballot_sync(hmask, at(c) >= t) >> (lane & 16)) & 0xffffu;
   return lo + (__ffs(b) - 1);
+}
+
+// the same on the cell offsets: the first cell that starts at or after particle t
+__device__ __forceinline__ int64_t lower_bound16(const int64_t *__restrict__ off, int64_t n, int64_t t, int lane) {
+  return lower_bound16_by([=](int64_t c) { return off[c]; }, n, t, lane);
 }
 
 }  // namespace fpc
