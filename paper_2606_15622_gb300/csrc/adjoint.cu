@@ -10,13 +10,16 @@
 // Kernel 1 (one thread per cell, FP64): lambda from the forward solve's
 // stored factors (two triangular solves) or, without them, by re-assembling
 // A and eliminating A^T with partial pivoting; then -lambda is propagated
-// back through the assembly formulas by hand-written reverse mode.  Kernel 2 (four consecutive cells per warp, their particles
-// walked flat by all lanes): the per-particle polynomial above, in the
-// velocity's precision, one pass over the particles.
+// back through the assembly formulas by hand-written reverse mode.  Kernel 2
+// (equal slices of the particles, 32 cells' tables at a time): the
+// per-particle polynomial above, in the velocity's precision, one pass over
+// the particles.
+#include <climits>
 #include <cstdint>
 
 #include "closure_math.cuh"
 #include "fp_device.cuh"
+#include "quads.cuh"
 
 namespace fpc {
 
@@ -217,10 +220,253 @@ __global__ void __launch_bounds__(128, 4) adjoint_cell_kernel(const double *__re
 // ---------------------------------------------------------------------------
 // particle gradient
 // ---------------------------------------------------------------------------
+constexpr int kAConst = 40;         // table entries per cell
+constexpr int64_t kACellWork = 50;  // a cell's share of building a chunk's table, in particles (24: 98 us, 100: 98, 50: 94)
+
+// Per-cell table of the particle polynomial, every coefficient already
+// divided by N and with its multiplicity.  With c = v - U, r2 = |c|^2 and
+//   s_d = W_d . c + r2 z_d,    t = c . s + 3 r2 (z . c)
+//   dL/dv_d = B_d + sum_j c_j (Mu_dj + sum_{k >= j} A_{d,jk} c_k) + c_d t + r2 s_d
+// (Mu from gm_u and gm_theta, A from gm_u3, W from gm_w, z from gm_z;
+// B = gm_U / N minus the cell mean of the rest).
+enum { AA3 = 0, AW = 18, AZ = 24, AMU = 28, AU = 34, AB = 37 };
+
+// One cell's table row by one lane, from its moment gradients (first half)
+// and its moments (second half) staged in T.
+template <typename T>
+struct ParticleRow {
+  T inv_n, Mu[6], B[3];
+
+  __device__ __forceinline__ void gradients(const T *gc, int n, T *row) {
+    inv_n = n > 0 ? T(1) / T(n) : T(0);
+    T r[28];
+    // d/dc_d of the slot's monomial: 3 c^2 (111), 2 c_j c_k and c_j^2 (112), c_j c_k (123)
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+#pragma unroll
+        for (int k = j; k < 3; ++k)
+          r[AA3 + 6 * d + sym2(j, k)] = T(1 + (j == d) + (k == d)) * (gc[kU3 + sym3(d, j, k)] * inv_n);
+#pragma unroll
+    for (int s = 0; s < 6; ++s) {
+      const bool diag = s == 0 || s == 3 || s == 5;
+      r[AW + s] = (diag ? T(2) : T(1)) * (gc[kW + s] * inv_n);
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) r[AZ + d] = gc[kZ + d] * inv_n;
+    r[27] = T(0);
+    store_row(row, r);
+    const T gth = gc[kTheta] * inv_n * T(2.0 / 3.0);
+#pragma unroll
+    for (int s = 0; s < 6; ++s) {
+      const bool diag = s == 0 || s == 3 || s == 5;
+      Mu[s] = diag ? tfma(T(2), gc[kU2 + s] * inv_n, gth) : gc[kU2 + s] * inv_n;
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) B[d] = gc[kU + d] * inv_n;
+  }
+
+  // B less the cell mean of the polynomial, from the moments
+  __device__ __forceinline__ void moments(const T *mc, T *row) {
+    T u3[10], b[3];
+#pragma unroll
+    for (int s = 0; s < 10; ++s) u3[s] = mc[kU3 + s];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) b[i] = u3[sym3(i, 0, 0)] + u3[sym3(i, 1, 1)] + u3[sym3(i, 2, 2)];
+    T s4 = T(0);
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+#pragma unroll
+      for (int k = j; k < 3; ++k) {
+        const T u = mc[kU2 + sym2(j, k)], w = mc[kW + sym2(j, k)];
+        const T Wjk = row[AW + sym2(j, k)] * (j == k ? T(1) : T(2));
+        if (j == k) s4 += w;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          B[d] = tfma(-row[AA3 + 6 * d + sym2(j, k)], u, B[d]);
+          B[d] = tfma(-Wjk, u3[sym3(d, j, k)], B[d]);
+        }
+        B[j] = tfma(T(-4) * row[AZ + k], w, B[j]);
+        if (j != k) B[k] = tfma(T(-4) * row[AZ + j], w, B[k]);
+      }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) B[d] = tfma(-row[AW + sym2(d, j)], b[j], B[d]);
+      B[d] = tfma(-s4, row[AZ + d], B[d]);
+    }
+    const T r[12] = {Mu[0], Mu[1], Mu[2], Mu[3], Mu[4], Mu[5], mc[kU], mc[kU + 1], mc[kU + 2], B[0], B[1], B[2]};
+    store_row(row + AMU, r);
+  }
+};
+
+// Every warp of a resident grid takes an equal share of the work and walks its
+// cells in chunks of up to 32: lane l builds the table row of the
+// chunk's cell l, then the warp streams the chunk's particles in quads of
+// four consecutive ones, with vector loads and stores where the arrays'
+// alignment allows, the next quad loaded while one is computed, and one table
+// row loaded a quad (another where a quad crosses a cell).  Bound: FP32 by the
+// loads in flight and the tables' building (11.9M particles of 131,072 cells
+// 114 us with a 44-entry row and three 4-byte loads a particle, 83 now; 288 MB
+// at the copy rate: 42); FP64 by its pipe, 59 operations a particle (75
+// before, and the table was built eight lanes a cell): 819,200 particles
+// 212 -> 107 us (the operations alone: 96).  Registers: FP32 96 or 168 a
+// thread 102 / 92 us, FP64 168 a thread 112.
+template <typename VT>
+__global__ void __launch_bounds__(sizeof(VT) == 4 ? 128 : 64, 4)
+    adjoint_particle_kernel(const VT *__restrict__ v, int64_t np, const int64_t *__restrict__ off, int64_t n_cells,
+                            const double *__restrict__ mom, const double *__restrict__ gm, VT *__restrict__ gv,
+                            int vec) {
+  using T = VT;
+  constexpr int kW = sizeof(VT) == 4 ? 4 : 2;     // warps per block
+  constexpr int kRow = sizeof(VT) == 4 ? 44 : 42;  // table row stride: 16-byte accesses of eight rows hit all banks
+  constexpr int kIn = FP_NMOM | 1;
+  __shared__ __align__(16) T table[kW][32 * kRow];
+  __shared__ T stages[kW][32 * kIn];
+  __shared__ int cofs[kW][33];  // the chunk's cell starts, relative to its first particle
+  const int lane = threadIdx.x & 31;
+  const int wib = threadIdx.x >> 5;
+  const uint32_t warp = blockIdx.x * kW + wib, nwarps = gridDim.x * kW;
+  T *tab = table[wib], *stage = stages[wib];
+  int *co = cofs[wib];
+  const Share sh = warp_share(off, n_cells, kACellWork, warp, nwarps, lane);
+  const int64_t tA = sh.p0, tB = sh.p1, cb = sh.c1;
+
+  for (int64_t cbase = sh.first; cbase < cb; cbase += 32) {
+    const int64_t c = cbase + lane;
+    const bool valid = c < cb;
+    const int64_t a0 = off[valid ? c : cb];
+    const int64_t a1 = valid ? off[c + 1] : a0;
+    // the chunk's particle range, clipped to the slice
+    const int64_t o0 = max(__shfl_sync(0xffffffffu, a0, 0), tA);
+    const int64_t oe = min(__shfl_sync(0xffffffffu, a1, 31), tB);
+    const int i4 = (int)max(oe - o0, (int64_t)0);
+    co[lane] = (int)min(max(a0 - o0, (int64_t)0), (int64_t)i4);
+    if (lane == 31) co[32] = i4;
+    // ---- the chunk's particles, in quads (quad Q: particles 4Q .. 4Q + 3) ----
+    const int64_t Qs = o0 >> 2, Qe = i4 > 0 ? (o0 + i4 + 3) >> 2 : Qs;
+    const VT *px = v + o0, *py = px + np, *pz = py + np;
+    VT *qx = gv + o0, *qy = qx + np, *qz = qy + np;
+    // (a lane's first quad is loaded before the table is built, the next ones
+    // each while one is computed)
+    T nx[4], ny[4], nz[4];
+    auto load = [&](int qb) {
+      if (qb >= 0 && qb + 4 <= i4) {
+        load_comp(px + qb, vec & 3, nx);
+        load_comp(py + qb, (vec >> 2) & 3, ny);
+        load_comp(pz + qb, (vec >> 4) & 3, nz);
+      } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int q = qb + u;
+          nx[u] = ny[u] = nz[u] = T(0);
+          if ((unsigned)q < (unsigned)i4) {
+            nx[u] = px[q];
+            ny[u] = py[q];
+            nz[u] = pz[q];
+          }
+        }
+      }
+    };
+    const int qe = (int)((Qe << 2) - o0);
+    int qb = (int)(((Qs + lane) << 2) - o0);  // chunk index of the quad's first particle
+    if (qb < qe) load(qb);
+    {
+      const int ncell = (int)min(cb - cbase, (int64_t)32);
+      ParticleRow<T> r;
+      const bool both = ncell <= 16;  // both sets of rows fit the stage at once
+      stage_rows<FP_NMOM>(gm + cbase * FP_NMOM, ncell, stage, lane, both ? mom + cbase * FP_NMOM : nullptr, 16 * kIn);
+      __syncwarp();
+      if (valid) r.gradients(stage + lane * kIn, (int)(a1 - a0), tab + lane * kRow);
+      if (!both) {
+        __syncwarp();
+        stage_rows<FP_NMOM>(mom + cbase * FP_NMOM, ncell, stage, lane);
+        __syncwarp();
+      }
+      if (valid) r.moments(stage + (lane + (both ? 16 : 0)) * kIn, tab + lane * kRow);
+    }
+    __syncwarp();
+    for (; qb < qe; qb += 128) {
+      const bool whole = qb >= 0 && qb + 4 <= i4;
+      T mx[4], my[4], mz[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        mx[u] = nx[u];
+        my[u] = ny[u];
+        mz[u] = nz[u];
+      }
+      if (qb + 128 < qe) load(qb + 128);
+      // cell of the quad's first particle: the last cl with co[cl] <= max(qb, 0)
+      const int q0 = max(qb, 0);
+      int cl = 0;
+#pragma unroll
+      for (int st = 16; st >= 1; st >>= 1)
+        if (co[cl + st] <= q0) cl += st;
+      T K[kAConst];
+      load_row(tab + cl * kRow, K);
+      int next = cl < 31 ? co[cl + 1] : INT_MAX;  // where the next cell starts
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        // (particles outside the chunk are computed on zeros and not stored)
+        const int q = qb + u;
+        if (q >= next) {  // past a cell boundary (and any empty cells)
+          while (cl < 31 && co[cl + 1] <= q) ++cl;
+          load_row(tab + cl * kRow, K);
+          next = cl < 31 ? co[cl + 1] : INT_MAX;
+        }
+        const T cc[3] = {mx[u] - K[AU], my[u] - K[AU + 1], mz[u] - K[AU + 2]};
+        const T r2 = tfma(cc[0], cc[0], tfma(cc[1], cc[1], cc[2] * cc[2]));
+        T s[3], out[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          s[d] = r2 * K[AZ + d];
+#pragma unroll
+          for (int j = 0; j < 3; ++j) s[d] = tfma(K[AW + sym2(d, j)], cc[j], s[d]);
+        }
+        const T zc = tfma(K[AZ], cc[0], tfma(K[AZ + 1], cc[1], K[AZ + 2] * cc[2]));
+        const T t = tfma(T(3) * r2, zc, tfma(cc[0], s[0], tfma(cc[1], s[1], cc[2] * s[2])));
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          T g = K[AB + d];
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            T h = K[AMU + sym2(d, j)];
+#pragma unroll
+            for (int k = j; k < 3; ++k) h = tfma(K[AA3 + 6 * d + sym2(j, k)], cc[k], h);
+            g = tfma(cc[j], h, g);
+          }
+          out[d] = tfma(r2, s[d], tfma(cc[d], t, g));
+        }
+        mx[u] = out[0];
+        my[u] = out[1];
+        mz[u] = out[2];
+      }
+      if (whole) {
+        store_comp(qx + qb, vec & 3, mx);
+        store_comp(qy + qb, (vec >> 2) & 3, my);
+        store_comp(qz + qb, (vec >> 4) & 3, mz);
+      } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int q = qb + u;
+          if ((unsigned)q < (unsigned)i4) {
+            qx[q] = mx[u];
+            qy[q] = my[u];
+            qz[q] = mz[u];
+          }
+        }
+      }
+    }
+    __syncwarp();  // the table and offsets are rewritten by the next chunk
+  }
+}
+
+// ---- small problems ----
 constexpr int kAG = 8;              // lanes per cell while building constants
 constexpr int kACells = 32 / kAG;   // consecutive cells per warp task
 constexpr int kAWarps = 8;          // warps per block
-constexpr int kAConst = 44;         // table entries per cell
+constexpr int kAGConst = 44;        // table entries per cell
 
 // Per-cell table of the particle polynomial, every coefficient already
 // multiplied by 1/N and by its constant factor:
@@ -228,7 +474,7 @@ constexpr int kAConst = 44;         // table entries per cell
 //             + c_d (c.W'c + |c|^2 gz'.c) + |c|^2 (W'c)_d + |c|^4 gz''_d + B_d
 // with Mu' = Mu/N, A3'_{d,jk} = 3 m_jk A_{djk}/N (m = 1 on, 2 off the
 // diagonal), W' = 2W/N, gz' = 4gz/N, gz'' = gz/N, B = (gm_U - <grad psi>)/N.
-enum { AU = 0, AMU = 3, AA3 = 9, AW = 27, AGZ4 = 33, AGZ1 = 36, AB = 39 };
+enum { GU = 0, GMU = 3, GA3 = 9, GW = 27, GGZ4 = 33, GGZ1 = 36, GB = 39 };
 
 template <typename T>
 __device__ __forceinline__ T shfl_g(T x, int src, int lane) {
@@ -238,20 +484,22 @@ __device__ __forceinline__ T shfl_g(T x, int src, int lane) {
 // multiplicity of a symmetric third-order slot (111: 1, 112: 3, 123: 6)
 __host__ __device__ constexpr int mult3(int s) { return (s == 0 || s == 6 || s == 9) ? 1 : (s == 4 ? 6 : 3); }
 
+// FP32 particles of small problems: a warp takes four consecutive cells; an
+// 8-lane group folds its cell's moments and moment gradients into the 35
+// coefficients of the per-particle polynomial (shared-memory table), then all
+// 32 lanes walk the four cells' contiguous particle range.
 // A warp takes four consecutive cells; an 8-lane group folds its cell's
 // moments and moment gradients into the 35 coefficients of the per-particle
 // polynomial (shared-memory table), then all 32 lanes walk the four cells'
 // contiguous particle range.
-template <typename VT>
-__global__ void __launch_bounds__(32 * kAWarps, sizeof(VT) == 4 ? 3 : 1) adjoint_particle_kernel(const VT *__restrict__ v, int64_t np,
-                                                                        const int64_t *__restrict__ off,
-                                                                        int64_t n_cells,
-                                                                        const double *__restrict__ mom,
-                                                                        const double *__restrict__ gm,
-                                                                        VT *__restrict__ gv) {
-  using T = VT;
+__global__ void __launch_bounds__(32 * kAWarps, 3)
+    adjoint_particle_group_kernel(const float *__restrict__ v, int64_t np, const int64_t *__restrict__ off,
+                                  int64_t n_cells, const double *__restrict__ mom, const double *__restrict__ gm,
+                                  float *__restrict__ gv) {
+  using VT = float;
+  using T = float;
   constexpr int G = kAG;
-  __shared__ __align__(16) T table[kAWarps][kACells][kAConst];
+  __shared__ __align__(16) T table[kAWarps][kACells][kAGConst];
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
   const int lg = lane & (G - 1);
@@ -260,7 +508,7 @@ __global__ void __launch_bounds__(32 * kAWarps, sizeof(VT) == 4 ? 3 : 1) adjoint
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const VT *vx = v, *vy = v + np, *vz = v + 2 * np;
   VT *gx = gv, *gy = gv + np, *gz = gv + 2 * np;
-  T(*tab)[kAConst] = table[wib];
+  T(*tab)[kAGConst] = table[wib];
 
   for (int64_t base = warp * kACells; base < n_cells; base += nwarps * kACells) {
     const int64_t c = base + g;
@@ -336,31 +584,31 @@ __global__ void __launch_bounds__(32 * kAWarps, sizeof(VT) == 4 ? 3 : 1) adjoint
       const T gU0 = GM(kU) * inv_n, gU1 = GM(kU + 1) * inv_n, gU2 = GM(kU + 2) * inv_n;
       if (lg == 0) {
         T *r = tab[g];
-        r[AU] = U0;
-        r[AU + 1] = U1;
-        r[AU + 2] = U2;
+        r[GU] = U0;
+        r[GU + 1] = U1;
+        r[GU + 2] = U2;
 #pragma unroll
-        for (int s = 0; s < 6; ++s) r[AMU + s] = Mu[s] * inv_n;
+        for (int s = 0; s < 6; ++s) r[GMU + s] = Mu[s] * inv_n;
 #pragma unroll
         for (int d = 0; d < 3; ++d)
 #pragma unroll
           for (int j = 0; j < 3; ++j)
 #pragma unroll
             for (int k = j; k < 3; ++k)
-              r[AA3 + 6 * d + sym2(j, k)] = A3[sym3(d, j, k)] * (j == k ? T(3) : T(6)) * inv_n;
+              r[GA3 + 6 * d + sym2(j, k)] = A3[sym3(d, j, k)] * (j == k ? T(3) : T(6)) * inv_n;
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
-          for (int j = i; j < 3; ++j) r[AW + sym2(i, j)] = T(2) * W[i][j] * inv_n;
+          for (int j = i; j < 3; ++j) r[GW + sym2(i, j)] = T(2) * W[i][j] * inv_n;
         const T gUv[3] = {gU0, gU1, gU2};
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-          r[AGZ4 + d] = T(4) * gzv[d] * inv_n;
-          r[AGZ1 + d] = gzv[d] * inv_n;
-          r[AB + d] = gUv[d] - G0[d] * inv_n;
+          r[GGZ4 + d] = T(4) * gzv[d] * inv_n;
+          r[GGZ1 + d] = gzv[d] * inv_n;
+          r[GB + d] = gUv[d] - G0[d] * inv_n;
         }
-        r[AB + 3] = T(0);
-        r[AB + 4] = T(0);
+        r[GB + 3] = T(0);
+        r[GB + 4] = T(0);
       }
     }
     const int64_t o0 = __shfl_sync(0xffffffffu, a0, 0);
@@ -374,9 +622,9 @@ __global__ void __launch_bounds__(32 * kAWarps, sizeof(VT) == 4 ? 3 : 1) adjoint
 #pragma unroll 2
     for (int q = lane; q < i4; q += 32) {
       const int cl = (q >= i1) + (q >= i2) + (q >= i3);
-      T K[kAConst];
+      T K[kAGConst];
       load_row(tab[cl], K);
-      const T cc[3] = {px[q] - K[AU], py[q] - K[AU + 1], pz[q] - K[AU + 2]};
+      const T cc[3] = {px[q] - K[GU], py[q] - K[GU + 1], pz[q] - K[GU + 2]};
       // the six products c_j c_k (j <= k), in sym2 order
       const T pr[6] = {cc[0] * cc[0], cc[0] * cc[1], cc[0] * cc[2], cc[1] * cc[1], cc[1] * cc[2], cc[2] * cc[2]};
       const T r2 = pr[0] + pr[3] + pr[5];
@@ -384,16 +632,16 @@ __global__ void __launch_bounds__(32 * kAWarps, sizeof(VT) == 4 ? 3 : 1) adjoint
       T Wc[3];
 #pragma unroll
       for (int i = 0; i < 3; ++i)
-        Wc[i] = K[AW + sym2(i, 0)] * cc[0] + K[AW + sym2(i, 1)] * cc[1] + K[AW + sym2(i, 2)] * cc[2];
+        Wc[i] = K[GW + sym2(i, 0)] * cc[0] + K[GW + sym2(i, 1)] * cc[1] + K[GW + sym2(i, 2)] * cc[2];
       const T t = cc[0] * Wc[0] + cc[1] * Wc[1] + cc[2] * Wc[2] +
-                  r2 * (K[AGZ4] * cc[0] + K[AGZ4 + 1] * cc[1] + K[AGZ4 + 2] * cc[2]);
+                  r2 * (K[GGZ4] * cc[0] + K[GGZ4 + 1] * cc[1] + K[GGZ4 + 2] * cc[2]);
       T out[3];
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
-        T gd = K[AMU + sym2(d, 0)] * cc[0] + K[AMU + sym2(d, 1)] * cc[1] + K[AMU + sym2(d, 2)] * cc[2];
+        T gd = K[GMU + sym2(d, 0)] * cc[0] + K[GMU + sym2(d, 1)] * cc[1] + K[GMU + sym2(d, 2)] * cc[2];
 #pragma unroll
-        for (int s = 0; s < 6; ++s) gd += K[AA3 + 6 * d + s] * pr[s];
-        out[d] = gd + cc[d] * t + r2 * Wc[d] + r4 * K[AGZ1 + d] + K[AB + d];
+        for (int s = 0; s < 6; ++s) gd += K[GA3 + 6 * d + s] * pr[s];
+        out[d] = gd + cc[d] * t + r2 * Wc[d] + r4 * K[GGZ1 + d] + K[GB + d];
       }
       qx[q] = out[0];
       qy[q] = out[1];
@@ -414,6 +662,43 @@ static int adj_sm_count() {
   return n;
 }
 
+// FP32 calls on up to this many cells take the group kernel: a table of four
+// cells by eight lanes each is ready sooner than one of 32 by a lane each, and
+// its small footprint runs beside other streams' kernels (16,384 cells of 50
+// particles 11.9 us against 12.4, of 150 25.3 against 19.8; as a chunk of the
+// host-resident step 26.6 against 31; 40,000 cells of 50: 25.0 against 24.1)
+constexpr int64_t kGroupCells = 32768;
+
+// A persistent grid (fewer blocks for small problems: two cells a warp at
+// least).
+template <typename VT>
+static void launch_adjoint_particles(const VT *v, int64_t np, const int64_t *off, int64_t n_cells, const double *mom,
+                                     const double *gm, VT *gv, cudaStream_t st) {
+  if (sizeof(VT) == 4 && n_cells <= kGroupCells) {
+    const int64_t cells_per_block = kAWarps * kACells, cap = (int64_t)adj_sm_count() * 8;
+    int64_t blocks = (n_cells + cells_per_block - 1) / cells_per_block;
+    if (blocks > cap) blocks = cap;
+    adjoint_particle_group_kernel<<<(unsigned)blocks, 32 * kAWarps, 0, st>>>((const float *)v, np, off, n_cells, mom,
+                                                                              gm, (float *)gv);
+    return;
+  }
+  constexpr int kW = sizeof(VT) == 4 ? 4 : 2;
+  static int per_sm = 0;
+  if (!per_sm) {
+    int k = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, adjoint_particle_kernel<VT>, 32 * kW, 0) != cudaSuccess ||
+        k < 1)
+      k = 1;
+    per_sm = k;
+  }
+  int64_t blocks = (int64_t)adj_sm_count() * per_sm;
+  const int64_t by_cells = (n_cells + 2 * kW - 1) / (2 * kW);
+  if (blocks > by_cells) blocks = by_cells;
+  if (blocks < 1) blocks = 1;
+  adjoint_particle_kernel<VT>
+      <<<(unsigned)blocks, 32 * kW, 0, st>>>(v, np, off, n_cells, mom, gm, gv, quad_classes(v, gv, np, 0, sizeof(VT)));
+}
+
 void launch_adjoint(const void *v, int v_dtype, int64_t np, const int64_t *off, int64_t n_cells, const double *tau,
                     double eps2_hat, const double *mom, const double *coeffs, const int32_t *flags, const double *lu,
                     const double *gY, const double *gm_in, double *gm_out, void *gv, cudaStream_t st) {
@@ -429,18 +714,10 @@ void launch_adjoint(const void *v, int v_dtype, int64_t np, const int64_t *off, 
                                                                        n_cells, eps2_hat, gm_out);
   }
   if (!gv) return;
-  const int threads = 32 * kAWarps;
-  const int64_t cells_per_block = kAWarps * kACells;
-  int64_t blocks = (n_cells + cells_per_block - 1) / cells_per_block;
-  const int64_t cap = (int64_t)adj_sm_count() * 8;
-  if (blocks > cap) blocks = cap;
-  if (blocks < 1) blocks = 1;
   if (v_dtype == FP_V_F32)
-    adjoint_particle_kernel<float><<<(unsigned)blocks, threads, 0, st>>>((const float *)v, np, off, n_cells, mom,
-                                                                         gm_out, (float *)gv);
+    launch_adjoint_particles<float>((const float *)v, np, off, n_cells, mom, gm_out, (float *)gv, st);
   else
-    adjoint_particle_kernel<double><<<(unsigned)blocks, threads, 0, st>>>((const double *)v, np, off, n_cells, mom,
-                                                                          gm_out, (double *)gv);
+    launch_adjoint_particles<double>((const double *)v, np, off, n_cells, mom, gm_out, (double *)gv, st);
 }
 
 }  // namespace fpc

@@ -204,4 +204,19 @@ __device__ __forceinline__ void load_row(const double *__restrict__ row, double 
   }
 }
 
+// and back
+template <int NC>
+__device__ __forceinline__ void store_row(float *row, const float (&K)[NC]) {
+  static_assert(NC % 4 == 0, "row length");
+#pragma unroll
+  for (int q = 0; q < NC / 4; ++q)
+    reinterpret_cast<float4 *>(row)[q] = make_float4(K[4 * q], K[4 * q + 1], K[4 * q + 2], K[4 * q + 3]);
+}
+template <int NC>
+__device__ __forceinline__ void store_row(double *row, const double (&K)[NC]) {
+  static_assert(NC % 2 == 0, "row length");
+#pragma unroll
+  for (int q = 0; q < NC / 2; ++q) reinterpret_cast<double2 *>(row)[q] = make_double2(K[2 * q], K[2 * q + 1]);
+}
+
 }  // namespace fpc

@@ -8,6 +8,21 @@
 
 namespace fpc {
 
+// Alignment classes of whole quads, per component (bits 2d, 2d + 1): quad Q
+// of component d starts at element d np + 4Q - first of two arrays based at
+// v and v_out (first: the elements by which particle 0 comes after a quad's
+// start)
+inline int quad_classes(const void *v, const void *v_out, int64_t np, int64_t first, size_t size) {
+  int vec = 0;
+  if ((uintptr_t)v % 16 || (uintptr_t)v_out % 16) return 0;
+  for (int d = 0; d < 3; ++d) {
+    const int e = (int)(((d * np - first % 4) % 4 + 4) % 4);
+    const int cls = size == 4 ? (e == 0 ? 2 : (e == 2 ? 1 : 0)) : (e % 2 == 0 ? 2 : 0);
+    vec |= cls << (2 * d);
+  }
+  return vec;
+}
+
 // a quad of one component by its alignment class (2: one 16-byte access of
 // floats or two of doubles, 1: two 8-byte float pairs, 0: four scalars)
 template <typename T>
@@ -69,6 +84,62 @@ __device__ __forceinline__ void store_comp<double>(double *p, int cls, const dou
     p[0] = x[0], p[1] = x[1], p[2] = x[2], p[3] = x[3];
 }
 
+// FP64 -> T for a table.  To FP32 on the integer pipe, to nearest even, values
+// below the smallest normal number to zero: the FP64 pipe takes 68 cycles a
+// conversion, this about 20 (values past FP32's range, which branch, aside).
+template <typename T>
+__device__ __forceinline__ T narrow(double x);
+template <>
+__device__ __forceinline__ double narrow<double>(double x) { return x; }
+template <>
+__device__ __forceinline__ float narrow<float>(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t a = hi & 0x7fffffffu;
+  // the top 23 fraction bits under the exponent less 896 (modulo 2^32)
+  uint32_t u = __funnelshift_l(lo, hi, 3) - (896u << 23);
+  u += ((lo & 0x1fffffffu) + 0x0fffffffu + (u & 1u)) >> 29;
+  u = (a < (897u << 20) ? 0u : u & 0x7fffffffu) | (hi & 0x80000000u);
+  float f = __uint_as_float(u);
+  if (__builtin_expect(a >= (1150u << 20), 0)) f = (float)x;
+  return f;
+}
+
+// Rows of NK doubles of up to 32 consecutive cells into shared memory as T,
+// row l at stage + l (NK | 1) (an odd stride: the lanes then read their own
+// rows without bank conflicts).  The warp's loads are contiguous; a lane that
+// read its own row from global memory would touch a line a load (32 wavefronts
+// an instruction).  The narrowing stays on the FP64 pipe, which these kernels
+// leave idle (d2f_rn's integers: 100 us against 83 for the adjoint's pass).
+// `more` (if not null): a second set of rows, loaded beside the first into
+// stage + more_at.
+template <int NK, typename T>
+__device__ __forceinline__ void stage_rows(const double *__restrict__ rows, int ncell, T *stage, int lane,
+                                           const double *__restrict__ more = nullptr, int more_at = 0) {
+  constexpr int kAt = 5;  // loads of a set in flight
+  const int total = ncell * NK;
+#pragma unroll 1
+  for (int t0 = 0; t0 * 32 < total; t0 += kAt) {
+    double x[kAt], y[kAt];
+#pragma unroll
+    for (int t = 0; t < kAt; ++t) {
+      const int i = (t0 + t) * 32 + lane;
+      if (i < total) {
+        x[t] = rows[i];
+        if (more) y[t] = more[i];
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < kAt; ++t) {
+      const int i = (t0 + t) * 32 + lane;
+      if (i < total) {
+        T *at = stage + i + ((NK | 1) - NK) * (i / NK);
+        *at = narrow<T>(x[t]);
+        if (more) at[more_at] = narrow<T>(y[t]);
+      }
+    }
+  }
+}
+
 // The first cell c in [0, n] with at(c) >= t (at nondecreasing, at(n) >= t),
 // found by the 16 lanes of the calling half warp together: each round probes
 // 16 evenly spaced cells and keeps the interval where the answer lies, so
@@ -102,6 +173,54 @@ __device__ __forceinline__ int64_t lower_bound16_by(At at, int64_t n, int64_t t,
 // the same on the cell offsets: the first cell that starts at or after particle t
 __device__ __forceinline__ int64_t lower_bound16(const int64_t *__restrict__ off, int64_t n, int64_t t, int lane) {
   return lower_bound16_by([=](int64_t c) { return off[c]; }, n, t, lane);
+}
+
+// Equal shares of a pass over the particles that also prepares every cell: the
+// work before particle p of cell c counts as p + kCell (c + 1), before the
+// preparation of cell c as off[c] + kCell c.  Share k of n: a warp's particles
+// [p0, p1), the cells [c0, c1) whose preparation falls in the share (those
+// that it owns), and first = c0 or, where the share starts inside a cell,
+// that cell.  (Shares equal in particles alone leave the warps of a rarefied
+// region, with ten times the cells, running long after the others.)
+struct Share {
+  int64_t p0, p1, c0, c1, first;
+};
+// (n <= 2^14.  Below 2^32 the shares come from 32-bit divisions: a 64-bit one is
+// some hundred instructions in a row.)
+__device__ __forceinline__ Share warp_share(const int64_t *__restrict__ off, int64_t n_cells, int64_t kCell, uint32_t k,
+                                            uint32_t n, int lane) {
+  if (n_cells <= 8 * (int64_t)n) {
+    // a few whole cells a share: no search (its dependent loads take 3 us);
+    // the cells' own offsets bound the particles
+    Share s;
+    s.c0 = s.first = (int64_t)((uint32_t)n_cells * k / n);
+    s.c1 = (int64_t)((uint32_t)n_cells * (k + 1) / n);
+    s.p0 = INT64_MIN;
+    s.p1 = INT64_MAX;
+    return s;
+  }
+  const int64_t base = off[0], total = off[n_cells] - base + kCell * n_cells;
+  const uint32_t kk = lane < 16 ? k : k + 1;
+  const int64_t t = base + (total >> 32 == 0 ? (int64_t)((uint32_t)total / n) * kk + (uint32_t)total % n * kk / n
+                                             : total / n * kk + total % n * kk / n);
+  int64_t c = lower_bound16_by([=](int64_t i) { return off[i] + kCell * i; }, n_cells, t, lane);
+  // t lies in cell c - 1: in its preparation (the cell goes to the next share)
+  // or among its particles
+  int64_t p = off[c];
+  if (c > 0) {
+    const int64_t q = t - kCell * c;
+    if (q <= off[c - 1])
+      p = off[--c];
+    else if (q < p)
+      p = q;
+  }
+  Share s;
+  s.p0 = __shfl_sync(0xffffffffu, p, 0);
+  s.p1 = __shfl_sync(0xffffffffu, p, 16);
+  s.c0 = __shfl_sync(0xffffffffu, c, 0);
+  s.c1 = __shfl_sync(0xffffffffu, c, 16);
+  s.first = s.c0 > 0 && off[s.c0] > s.p0 ? s.c0 - 1 : s.c0;
+  return s;
 }
 
 }  // namespace fpc

@@ -668,18 +668,7 @@ __global__ void __launch_bounds__(sizeof(VT) == 4 ? 256 : 128, sizeof(VT) == 4 ?
 
 static VelParams make_vel_params(double dt, double eps2_hat, uint64_t seed, uint64_t step, uint64_t poff,
                                  const void *v, const void *v_out, int64_t np, int v_dtype) {
-  int vec = 0;
-  if ((uintptr_t)v % 16 == 0 && (uintptr_t)v_out % 16 == 0) {
-    for (int d = 0; d < 3; ++d) {
-      const int e = (int)((((int64_t)d * np - (int64_t)(poff % 4)) % 4 + 4) % 4);  // element alignment
-      int cls = 0;
-      if (v_dtype == FP_V_F32)
-        cls = e == 0 ? 2 : (e == 2 ? 1 : 0);
-      else
-        cls = e % 2 == 0 ? 2 : 0;  // two 16-byte pairs cover a quad of doubles
-      vec |= cls << (2 * d);
-    }
-  }
+  const int vec = quad_classes(v, v_out, np, (int64_t)(poff % 4), v_dtype == FP_V_F32 ? 4 : 8);
   return VelParams{dt, eps2_hat, step, poff, philox_keys(seed), vec};
 }
 
