@@ -82,12 +82,13 @@ enum { FP_V_F32 = 0, FP_V_F64 = 1 };
  * The 9x9 system is assembled in FP64 in both modes and solved with partial
  * pivoting; the FP64 mode, and any call that keeps the factors for the
  * adjoint, eliminates in FP64.  Without factors the FP32-moment mode factors
- * the system in FP32 and refines the solution once against the FP64 residual
- * b - A x (agreeing with the FP64 elimination to ~1e-9 relative, far below
- * the moments' own error); cells whose FP32 pivots fall below
- * max(3e-3, 100 pivot_rtol) of max|A|, or whose correction exceeds 1e-4 of
- * the solution, are eliminated in FP64 instead, and that elimination decides
- * their flags.  With FP32
+ * the system in FP32 and refines the solution once against the residual
+ * b - A x, formed in pairs of FP32 numbers (~46 bits; agreeing with the FP64
+ * elimination to ~1e-9 relative, far below the moments' own error); cells
+ * whose FP32 pivots fall below max(3e-3, 100 pivot_rtol) of max|A|, whose
+ * correction exceeds 1e-4 of the solution, or whose theta or tau lies beyond
+ * 2^+-20, are eliminated in FP64 instead, and that elimination decides their
+ * flags.  With FP32
  * moments (relative error ~1e-7) a pivot below ~1e-6 max|A| cannot be told
  * from zero, so that mode flags a cell singular when a pivot is
  * <= max(pivot_rtol, FP_FP32_PIVOT_FLOOR) * max|A|.  A cell of four

@@ -202,20 +202,102 @@ __global__ void __launch_bounds__(256) gather_fp32_kernel(const VT *__restrict__
 // the whole register file, and the third of the file it leaves free lets the
 // learned closure's kernels run beside it in the step.  With kLU the factors
 // of P A = L U of every unflagged cell go to lu for the adjoint.
-template <bool kLU, bool kMixed = false>
+template <bool kLU>
 __global__ void __launch_bounds__(128, 3) solve_kernel(const double *__restrict__ mom, const double *__restrict__ tau,
                                                        int64_t n_cells, SolveParams prm, double *__restrict__ coeffs,
                                                        int32_t *__restrict__ flags, double *__restrict__ lu) {
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n_cells;
        c += (int64_t)gridDim.x * blockDim.x) {
     double y[9];
-    const int fl = kMixed ? closure_cell_mixed(mom + c * FP_NMOM, tau[c], prm, y)
-                          : closure_cell<kLU>(mom + c * FP_NMOM, tau[c], prm, y, kLU ? lu + lu_base(c) : nullptr);
+    const int fl = closure_cell<kLU>(mom + c * FP_NMOM, tau[c], prm, y, kLU ? lu + lu_base(c) : nullptr);
     double *yc = coeffs + c * 9;
 #pragma unroll
     for (int q = 0; q < 9; ++q) yc[q] = y[q];
     flags[c] = fl;
   }
+}
+
+// The FP64 elimination of the cells of `todo` (a bit a lane; cell c0 + lane) by
+// the whole warp, two at a time, a half warp each: the same results as a
+// thread's in half the time, and one late cell does not hold up its warp for
+// a whole single-lane elimination (25 us).  Out of line: its registers are not
+// the mixed path's.
+static __device__ __noinline__ void solve_listed(unsigned todo, int64_t c0, const double *__restrict__ mom,
+                                                 const double *__restrict__ tau, const SolveParams &prm,
+                                                 double *__restrict__ coeffs, int32_t *__restrict__ flags) {
+  const int lane = threadIdx.x & 31, r = lane & 15;
+  while (todo) {
+    const int first = __ffs(todo) - 1;
+    todo &= todo - 1;
+    const int second = todo ? __ffs(todo) - 1 : -1;
+    if (todo) todo &= todo - 1;
+    const int mine = lane < 16 ? first : second;
+    const bool valid = mine >= 0;
+    const int64_t c = c0 + (valid ? mine : first);
+    double y[9];
+    const int fl = closure_cell_group16(mom + c * FP_NMOM, tau[c], prm, valid, r, y);
+    if (valid && r == 0) {
+#pragma unroll
+      for (int q = 0; q < 9; ++q) coeffs[c * 9 + q] = y[q];
+      flags[c] = fl;
+    }
+  }
+}
+
+// and of a lane's own cell (where many of a warp's cells need it: a thread's
+// elimination costs the FP64 pipe as much as four by half warps, for up to 32)
+static __device__ __noinline__ void solve_own(int64_t c, const double *__restrict__ mom,
+                                              const double *__restrict__ tau, const SolveParams &prm,
+                                              double *__restrict__ coeffs, int32_t *__restrict__ flags) {
+  double y[9];
+  const int fl = closure_cell<false>(mom + c * FP_NMOM, tau[c], prm, y);
+#pragma unroll
+  for (int q = 0; q < 9; ++q) coeffs[c * 9 + q] = y[q];
+  flags[c] = fl;
+}
+
+// The mixed-precision solve, one thread per cell; cells that it refuses are
+// solved by their warp.  Three blocks per SM: bound by the dependent chains
+// of the FP32 elimination and the selects of its row swaps.
+// 131,072 cells of 91 particles: 70 us (97 with the residual in FP64 and a
+// single-lane fallback), 16,384 of 50: 29 (36.5);
+// two or four blocks per SM 75 / 72.
+__global__ void __launch_bounds__(128, 3) solve_mixed_kernel(const double *__restrict__ mom,
+                                                             const double *__restrict__ tau, int64_t n_cells,
+                                                             SolveParams prm, double *__restrict__ coeffs,
+                                                             int32_t *__restrict__ flags) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t c0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; c0 < n_cells;
+       c0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t c = c0 + lane;
+    bool todo = false;
+    if (c < n_cells) {
+      double y[9];
+      const int fl = closure_cell_mixed(mom + c * FP_NMOM, tau[c], prm, y, todo);
+      if (!todo) {
+        double *yc = coeffs + c * 9;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) yc[q] = y[q];
+        flags[c] = fl;
+      }
+    }
+    const unsigned list = __ballot_sync(0xffffffffu, todo);
+    if (__popc(list) > 4) {
+      if (todo) solve_own(c, mom, tau, prm, coeffs, flags);
+    } else if (list) {
+      solve_listed(list, c0, mom, tau, prm, coeffs, flags);
+    }
+  }
+}
+
+// The FP64 solve of few cells, a half warp a cell (the same results as
+// solve_kernel's).
+__global__ void __launch_bounds__(128) solve_group_kernel(const double *__restrict__ mom,
+                                                          const double *__restrict__ tau, int64_t n_cells,
+                                                          SolveParams prm, double *__restrict__ coeffs,
+                                                          int32_t *__restrict__ flags) {
+  const int64_t c0 = 2 * (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  if (c0 < n_cells) solve_listed(c0 + 1 < n_cells ? 3u : 1u, c0, mom, tau, prm, coeffs, flags);
 }
 
 // ---------------------------------------------------------------------------
@@ -268,14 +350,21 @@ void launch_solve(const double *mom, const double *tau, int64_t n_cells, const f
   if (prec == FP_PREC_FP32_MOMENTS && rtol < FP_FP32_PIVOT_FLOOR) rtol = FP_FP32_PIVOT_FLOOR;
   SolveParams prm{p.eps2_hat, rtol, p.min_particles, prec == FP_PREC_FP32_MOMENTS ? FP_FP32_MIN_REGULAR : 0};
   const int threads = 128;
-  int64_t blocks = (n_cells + threads - 1) / threads;
-  if (blocks > 2 * sm_count()) blocks = 2 * sm_count();
+  const int64_t blocks = (n_cells + threads - 1) / threads;
+  const unsigned two = (unsigned)(blocks < 2 * sm_count() ? blocks : 2 * sm_count());
+  const unsigned three = (unsigned)(blocks < 3 * sm_count() ? blocks : 3 * sm_count());
+  // a half warp a cell while every SM sub-partition has one warp of them at
+  // most (eight times the FP64 instructions a cell, half the chain): 400 cells
+  // 16.5 us against 25.3
+  const bool few = n_cells <= 8 * (int64_t)sm_count();
   if (lu)
-    solve_kernel<true><<<(unsigned)blocks, threads, 0, st>>>(mom, tau, n_cells, prm, coeffs, flags, lu);
+    solve_kernel<true><<<two, threads, 0, st>>>(mom, tau, n_cells, prm, coeffs, flags, lu);
   else if (prec == FP_PREC_FP32_MOMENTS)  // FP32-accurate moments: the mixed-precision solve
-    solve_kernel<false, true><<<(unsigned)blocks, threads, 0, st>>>(mom, tau, n_cells, prm, coeffs, flags, nullptr);
+    solve_mixed_kernel<<<three, threads, 0, st>>>(mom, tau, n_cells, prm, coeffs, flags);
+  else if (few)
+    solve_group_kernel<<<(unsigned)((n_cells + 7) / 8), threads, 0, st>>>(mom, tau, n_cells, prm, coeffs, flags);
   else
-    solve_kernel<false><<<(unsigned)blocks, threads, 0, st>>>(mom, tau, n_cells, prm, coeffs, flags, nullptr);
+    solve_kernel<false><<<two, threads, 0, st>>>(mom, tau, n_cells, prm, coeffs, flags, nullptr);
 }
 
 }  // namespace fpc

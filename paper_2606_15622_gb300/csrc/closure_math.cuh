@@ -306,11 +306,10 @@ __device__ __forceinline__ int closure_cell(const double *__restrict__ mc, doubl
 
 // ---------------------------------------------------------------------------
 // Mixed-precision solve for FP32 moments: the system is factored in FP32 (on
-// the FP32 pipe), the residual b - A x is formed in FP64 straight from the
-// emitted entries (the FP64 matrix is never stored), and one correction solve
-// with the FP32 factors refines x.  Each FP64 instruction costs this GPU ~64
-// times an FP32 one, so this moves about three quarters of the FP64 work of
-// the plain solve off the FP64 pipe.  The refinement converges at a rate of
+// the FP32 pipe), the residual b - A x is formed in pairs of FP32 (below)
+// straight from the moments, and one correction solve with the FP32 factors
+// refines x.  Each FP64 instruction costs this GPU ~64 times an FP32 one; no
+// step of this path is one.  The refinement converges at a rate of
 // about kappa times the FP32 rounding of the system, and on an ill-conditioned
 // cell a small correction does not mean a small error, so a cell is refined
 // only if its smallest FP32 pivot is at least max(3e-3, 100 rtol) of max|A|
@@ -318,6 +317,145 @@ __device__ __forceinline__ int closure_cell(const double *__restrict__ mc, doubl
 // its correction is at most 1e-4 of x; any other cell is solved again by the
 // FP64 elimination, which then also decides its flags.
 // ---------------------------------------------------------------------------
+// A number as h + l, |l| about 2^-24 |h|: pairs of FP32 carry some 46 bits,
+// the residual of a solution whose own error is 2^-24 kappa needs about 40.
+struct F2 {
+  float h, l;
+};
+
+// double -> F2 on the integer pipe: the leading 24 bits truncated, the other 29
+// rounded to FP32.  For |x| < 2^100; below 2^-74 without the low bits, below
+// 2^-120 zero.
+__device__ __forceinline__ F2 f2_split(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t sign = hi & 0x80000000u, e = (hi >> 20) & 0x7ffu;
+  const bool tiny = e < 1023u - 120u;
+  F2 r;
+  r.h = __uint_as_float(tiny ? sign : ((__funnelshift_l(lo, hi, 3) - (896u << 23)) & 0x7fffffffu) | sign);
+  // the low 29 bits count 2^(e - 1075)
+  const float unit = __uint_as_float(e <= 1075u - 127u ? 0u : ((e - 1075u + 127u) << 23) | sign);
+  r.l = __uint2float_rn(lo & 0x1fffffffu) * unit;
+  return r;
+}
+__device__ __forceinline__ F2 f2_fast(float a, float b) {  // |a| >= |b|
+  const float s = a + b;
+  return F2{s, b - (s - a)};
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+  float s, e;
+  two_sum(a.h, b.h, s, e);
+  return f2_fast(s, e + (a.l + b.l));
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+  const float p = a.h * b.h;
+  return f2_fast(p, fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p))));
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, float b) {
+  const float p = a.h * b;
+  return f2_fast(p, fmaf(a.l, b, fmaf(a.h, b, -p)));
+}
+__device__ __forceinline__ F2 f2_scale(F2 a, float b) { return F2{a.h * b, a.l * b}; }  // b a power of two
+__device__ __forceinline__ F2 f2_recip(F2 a) {  // one Newton step from 1 / h
+  const float y = 1.f / a.h;
+  const float e = fmaf(-a.l, y, fmaf(-a.h, y, 1.f));
+  return f2_fast(y, y * e);
+}
+// (h, l) += a b without renormalising: h by two-sum, the rest into l
+__device__ __forceinline__ void f2_mac(F2 &s, F2 a, float b) {
+  const float p = a.h * b, e = fmaf(a.l, b, fmaf(a.h, b, -p));
+  float t, f;
+  two_sum(s.h, p, t, f);
+  s.h = t;
+  s.l += e + f;
+}
+__device__ __forceinline__ void f2_mac(F2 &s, F2 a, F2 b) {
+  const float p = a.h * b.h, e = fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p)));
+  float t, f;
+  two_sum(s.h, p, t, f);
+  s.h = t;
+  s.l += e + f;
+}
+
+// The residual of the moment-matching system (assemble_emit's rows) at
+// y = x[0..8], rounded to FP32: the rows' sums over the moments themselves,
+//   stress (ij):  -(2/tau) u_ij + 2 e2 w_ij
+//                 - [sum_k (C_ik u_kj + C_jk u_ki) + G_i b_j + G_j b_i]
+//   heat (i):     -(4/(3 tau)) b_i + e2 (3 z_i - 3 th b_i - 2 u_ik b_k)
+//                 - [sum_l C_il b_l + 2 sum_kl C_kl u_ikl + G_i (s4 - 9 th^2)
+//                    + 2 sum_k G_k w_ki - 6 th sum_k G_k u_ki]
+__device__ __forceinline__ void residual_f2(const double *__restrict__ mc, double tau, double eps2_hat,
+                                            const float (&x)[9], float (&res)[9]) {
+  F2 u[6], u3[10], w[6], b[3];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    u[q] = f2_split(mc[kU2 + q]);
+    w[q] = f2_split(mc[kW + q]);
+  }
+#pragma unroll
+  for (int q = 0; q < 10; ++q) u3[q] = f2_split(mc[kU3 + q]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) b[i] = f2_add(f2_add(u3[sym3(i, 0, 0)], u3[sym3(i, 1, 1)]), u3[sym3(i, 2, 2)]);
+  const F2 th = f2_split(mc[kTheta]), tc = f2_split(tau);
+  const F2 itau = f2_recip(tc);
+  const F2 e2 = f2_mul(f2_split(eps2_hat), f2_recip(f2_mul(tc, th)));
+  float n[9];  // -x
+#pragma unroll
+  for (int q = 0; q < 9; ++q) n[q] = -x[q];
+  const F2 mitau = F2{-itau.h, -itau.l};
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = i; j < 3; ++j) {
+      F2 s{0.f, 0.f};
+      f2_mac(s, u[sym2(i, j)], mitau);
+      f2_mac(s, w[sym2(i, j)], e2);
+      if (i == j) {  // half the row
+#pragma unroll
+        for (int k = 0; k < 3; ++k) f2_mac(s, u[sym2(k, i)], n[sym2(i, k)]);
+        f2_mac(s, b[i], n[6 + i]);
+        res[sym2(i, j)] = 2.f * (s.h + s.l);
+      } else {
+        s = f2_scale(s, 2.f);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          f2_mac(s, u[sym2(k, j)], n[sym2(i, k)]);
+          f2_mac(s, u[sym2(k, i)], n[sym2(j, k)]);
+        }
+        f2_mac(s, b[j], n[6 + i]);
+        f2_mac(s, b[i], n[6 + j]);
+        res[sym2(i, j)] = s.h + s.l;
+      }
+    }
+  const F2 th3 = f2_mul(th, 3.f);
+  F2 q4 = f2_add(f2_add(w[0], w[3]), w[5]);  // s4 - 9 theta^2
+  f2_mac(q4, th3, F2{-th3.h, -th3.l});
+  q4 = f2_fast(q4.h, q4.l);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    // half the row; its right-hand side first: -(2/3) b_i / tau + e2 (3/2 z_i - 3/2 th b_i - u_ik b_k)
+    F2 r{0.f, 0.f};
+    f2_mac(r, f2_split(mc[kZ + i]), 1.5f);
+    f2_mac(r, f2_mul(th3, -0.5f), b[i]);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) f2_mac(r, u[sym2(i, k)], F2{-b[k].h, -b[k].l});
+    F2 s{0.f, 0.f};
+    f2_mac(s, f2_fast(r.h, r.l), e2);
+    f2_mac(s, f2_mul(b[i], mitau), F2{0.666666687f, -1.98682148e-08f});  // 2/3
+    f2_mac(s, q4, 0.5f * n[6 + i]);
+    F2 g{0.f, 0.f};  // sum_k G_k u_ki
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      f2_mac(s, b[k], 0.5f * n[sym2(i, k)]);
+      f2_mac(s, w[sym2(k, i)], n[6 + k]);
+      f2_mac(g, u[sym2(k, i)], x[6 + k]);
+#pragma unroll
+      for (int l = k; l < 3; ++l) f2_mac(s, u3[sym3(i, k, l)], (k == l ? 1.f : 2.f) * n[sym2(k, l)]);
+    }
+    f2_mac(s, f2_fast(g.h, g.l), th3);
+    res[6 + i] = 2.f * (s.h + s.l);
+  }
+}
+
 template <int K>
 __device__ __forceinline__ void lu_step_f(float (&a)[9][10], float (&rinv)[9], uint64_t &perm, uint32_t &pmin) {
   uint32_t best = __float_as_uint(a[K][K]) & 0x7fffffffu;
@@ -393,31 +531,39 @@ __device__ __forceinline__ void lu_apply_f(const float (&a)[9][10], const float 
   }
 }
 
-// closure_cell in FP64 as a separate function, so that the rare fallback does
-// not add its registers to the mixed-precision path
-static __device__ __noinline__ int closure_cell_fp64(const double *__restrict__ mc, double tc, const SolveParams &prm,
-                                              double (&y)[9]) {
-  return closure_cell<false>(mc, tc, prm, y);
+// The linear drift C = -I/tau, G = 0 of a flagged cell
+__device__ __forceinline__ void linear_drift(double tc, double (&y)[9]) {
+  const double c0 = (finite_d(tc) && tc > 0.0) ? -1.0 / tc : 0.0;
+#pragma unroll
+  for (int q = 0; q < 9; ++q) y[q] = 0.0;
+  y[0] = c0;
+  y[3] = c0;
+  y[5] = c0;
 }
 
 // The closure of one cell from FP32-accurate moments by the mixed-precision
-// solve; flags and Y as closure_cell (which it falls back to).
+// solve; flags and Y as closure_cell.  todo: the cell needs the FP64
+// elimination (y and the flags are then not set).
 __device__ __forceinline__ int closure_cell_mixed(const double *__restrict__ mc, double tc, const SolveParams &prm,
-                                                  double (&y)[9]) {
+                                                  double (&y)[9], bool &todo) {
+  todo = false;
   int fl = 0;
+  bool in_range;  // of f2_split: theta and tau within 2^+-20, so z (order 5) within 2^+-50 of one
   {
-    double m[FP_NMOM];
-#pragma unroll
-    for (int k = 0; k < FP_NMOM; ++k) m[k] = mc[k];
     bool fin = finite_d(tc) && tc > 0.0;
 #pragma unroll
-    for (int k = 0; k < FP_NMOM; ++k) fin = fin && finite_d(m[k]);
+    for (int k = 0; k < FP_NMOM; ++k) fin = fin && finite_d(mc[k]);
     if (!fin) fl |= FP_FLAG_NONFINITE;
-    if (m[kN] < (double)prm.min_particles) fl |= FP_FLAG_FEW;
-    if (!(m[kTheta] > 0.0)) fl |= FP_FLAG_SINGULAR;
-    if (!fl && m[kN] < (double)prm.min_regular) fl |= FP_FLAG_SINGULAR;
+    if (mc[kN] < (double)prm.min_particles) fl |= FP_FLAG_FEW;
+    if (!(mc[kTheta] > 0.0)) fl |= FP_FLAG_SINGULAR;
+    if (!fl && mc[kN] < (double)prm.min_regular) fl |= FP_FLAG_SINGULAR;
+    auto near_one = [](double v) { return (((uint32_t)__double2hiint(v) >> 20) & 0x7ffu) - (1023u - 20u) < 40u; };
+    in_range = near_one(tc) && near_one(mc[kTheta]);
   }
-  if (fl) return closure_cell_fp64(mc, tc, prm, y);  // the linear drift, as there
+  if (fl) {
+    linear_drift(tc, y);
+    return fl;
+  }
   // FP32 system from the moments rounded to FP32 (integer pipe)
   float af[9][10];
   {
@@ -448,43 +594,24 @@ __device__ __forceinline__ int closure_cell_mixed(const double *__restrict__ mc,
   lu_step_f<7>(af, rinv, perm, pmin);
   lu_step_f<8>(af, rinv, perm, pmin);
   const float accept = fmaxf(3e-3f, (float)(100.0 * prm.pivot_rtol));
-  bool ok = amax < 0x7f800000u && __uint_as_float(pmin) > accept * __uint_as_float(amax);
+  bool ok = in_range && amax < 0x7f800000u && __uint_as_float(pmin) > accept * __uint_as_float(amax);
   if (ok) {
     back_sub_f(af, rinv, x0);
-    // residual b - A x0 in FP64 from the emitted entries
-    double x[9], res[9];
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-      x[q] = f2d_exact(x0[q]);
-      res[q] = 0.0;
-    }
-    {
-      double m[FP_NMOM];
-#pragma unroll
-      for (int k = 0; k < FP_NMOM; ++k) m[k] = mc[k];
-      assemble_emit(m, tc, prm.eps2_hat, [&](int row, int col, double v) {
-        if (col == 9)
-          res[row] += v;
-        else
-          res[row] = fma(-v, x[col], res[row]);
-      });
-    }
     float rf[9], d[9];
-#pragma unroll
-    for (int q = 0; q < 9; ++q) rf[q] = d2f_rn(res[q]);
+    residual_f2(mc, tc, prm.eps2_hat, x0, rf);
     lu_apply_f(af, rinv, perm, rf, d);
     float dmax = 0.f, xmax = 0.f;
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
       dmax = fmaxf(dmax, fabsf(d[q]));
       xmax = fmaxf(xmax, fabsf(x0[q]));
-      y[q] = x[q] + f2d_exact(d[q]);
+      y[q] = f2d_exact(x0[q]) + f2d_exact(d[q]);
     }
     ok = dmax <= 1e-4f * xmax;
 #pragma unroll
     for (int q = 0; q < 9; ++q) ok = ok && finite_d(y[q]);
   }
-  if (!ok) return closure_cell_fp64(mc, tc, prm, y);
+  todo = !ok;
   return 0;
 }
 
