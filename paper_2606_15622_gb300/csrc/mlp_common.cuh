@@ -53,17 +53,34 @@ __device__ __forceinline__ float silu_grad(float z) {
   return s * (1.f + z * (1.f - s));
 }
 
-// FP64 moment -> FP32 network input, rounded to nearest even (the hardware
-// conversion: the learned-closure kernels leave the FP64 pipe otherwise
-// idle, so it costs one issue slot where the integer-pipe version takes
-// about fifteen).
-__device__ __forceinline__ float narrow(double x) { return __double2float_rn(x); }
+// FP64 moment -> FP32 network input, rounded to nearest even.
+// Rounded on the integer pipes: a conversion on the FP64 pipe holds a
+// sub-partition 68 cycles a warp.  narrow_common is right for values whose
+// FP32 exponent is in the normal range (not above 2^127) and returns whether
+// x is one; narrow leaves the others to the conversion, zeros aside.
+__device__ __forceinline__ bool narrow_common(double x, float &f) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  // the top 23 fraction bits under the exponent less 896 (modulo 2^32), half to even on the 29 below
+  uint32_t u = __funnelshift_l(lo, hi, 3) - (896u << 23);
+  u += ((lo & 0x1fffffffu) + 0x0fffffffu + (u & 1u)) >> 29;
+  f = __uint_as_float((u & 0x7fffffffu) | (hi & 0x80000000u));
+  return (hi & 0x7fffffffu) - (897u << 20) < (253u << 20);
+}
+__device__ __forceinline__ float narrow(double x) {
+  float f;
+  if (!narrow_common(x, f)) f = (__double_as_longlong(x) << 1) == 0 ? __int_as_float(__double2hiint(x)) : __double2float_rn(x);
+  return f;
+}
 
 // standardisation of the network's inputs: x = (f - mu) * (1 / sigma)
 __device__ __forceinline__ float standardise(float f, float mu, float inv_sigma) { return (f - mu) * inv_sigma; }
 
-// The 16 raw inputs of one cell from its LITE vector and tau, in FP32.
-__device__ __forceinline__ void lite_raw_features(const double *__restrict__ m, double tau, float (&f)[16]) {
+__device__ __forceinline__ float narrow(float x) { return x; }  // (a vector narrowed beforehand)
+
+// The 16 raw inputs of one cell from its LITE vector (FP64, or narrowed) and
+// tau, in FP32.
+template <typename T>
+__device__ __forceinline__ void lite_raw_features(const T *__restrict__ m, double tau, float (&f)[16]) {
   const float th = narrow(m[4]);
   const float u00 = narrow(m[5]), u01 = narrow(m[6]), u02 = narrow(m[7]), u11 = narrow(m[8]), u12 = narrow(m[9]),
               u22 = narrow(m[10]);

@@ -10,8 +10,8 @@
 //     32 columns at a time with tcgen05.ld; bias, SiLU (through tanh) and
 //     BF16 rounding turn them into 32 columns of the next layer's A operand
 //     in shared memory;
-//   - after each 32-column chunk the group's leader issues the next layer's
-//     tcgen05.mma instructions over those 32 K-columns (M = 128, K = 16 each,
+//   - after every second 32-column chunk the group's leader issues the next
+//     layer's tcgen05.mma instructions over those 64 K-columns (M = 128, K = 16 each,
 //     N = 128, or 16 for the output layer) into the other accumulator buffer
 //     D[l + 1], so the tensor cores work while the epilogue continues, and
 //     commits the layer to the group's mbarrier after the last chunk;
@@ -30,14 +30,23 @@
 // r, pass k, layer l, column j uses word j % 4 of Philox4x32-10 (key = the
 // probe's seed) on counter (r lo, r hi, k, 32 l + j / 4): dropped when
 // (floor(w / 2^8) + 1) 2^-24 <= rate.
-// The learned closure runs as one instance of this kernel: the group's two
-// threads per row form the row's inputs from its moment (or LITE) vector
-// straight into the input tile -- the next tile's rows are bulk-prefetched
-// into L2 while the current tile runs, and formed once its last layer is
-// done -- and the output threads turn the predictions into coefficients,
+// The learned closure runs as one instance of this kernel: eight more warps
+// form the rows' inputs from the moment (or LITE) vectors straight into the
+// input tiles, and the output threads turn the predictions into coefficients,
 // check the energy residual, write the flags and append the cells that need
 // the exact closure to a list (one atomic per warp), so the inputs and the
-// predictions never travel through HBM.
+// predictions never travel through HBM.  The forming warps run one tile ahead
+// of each group: rows bulk-prefetched into L2 a tile before, staged in shared
+// memory as FP32 by contiguous loads, the features written once the first
+// layer has read the input tile, what the output layer needs of them once the
+// output layer has read the last tile's.
+// Bound by each group's chain of layers (MMA wait, tensor-memory loads, SiLU,
+// barrier), two groups in flight: tensor memory holds no third pair of
+// accumulators.  tanh alone is 115 us of 2^20 cells (8 cycles a warp), the
+// rows' bytes 50.  2^20 cells: 278 us; 395 with the inputs formed by the
+// groups' own threads between two tiles, 288 with four forming warps; 245
+// with nothing to stage.  Issuing the next layer's MMAs every 32 columns
+// 296, once a layer 276.
 // Only the group's leader waits on the mbarrier, with a bound, and passes its
 // outcome to the group through shared memory at the next group barrier; a
 // wait that runs out marks the group's remaining rows (NaN outputs, or
@@ -59,6 +68,7 @@ constexpr int kTcRows = 128;                 // rows per tile = TMEM lanes
 constexpr int kTcGroups = 2;                 // tiles in flight per CTA
 constexpr int kTcGroupThreads = 256;         // two threads per row: 16 of every 32 columns each
 constexpr int kTcThreads = kTcGroupThreads * kTcGroups;
+constexpr int kFormThreads = 256;            // closure variants: eight more warps form the next tiles' inputs
 constexpr uint32_t kTmemCols = 512;          // two 128-column accumulators per group
 
 // shared-memory carve-up (bytes from a 1024-byte aligned base)
@@ -72,8 +82,14 @@ constexpr uint32_t kNBias = 4 * kHid + 3 * kOut;               // b1..b4 / 2, b5
 constexpr uint32_t kOffBar = kOffBias + kNBias * 4;            // 2 mbarriers
 constexpr uint32_t kOffTmemSlot = kOffBar + 8 * kTcGroups;       // TMEM address + two outcomes
 constexpr uint32_t kOffScal = kOffTmemSlot + 16;               // [32] float4 input scalers (closure variants)
-constexpr uint32_t kOffFlags = kOffScal + 4 * kIn * 4;         // [2 groups][2 parities][128] part-1 input flags
-constexpr uint32_t kTcSmemUsed = kOffFlags + kTcGroups * 2 * kTcRows * 4;
+constexpr uint32_t kOffState = kOffScal + 4 * kIn * 4;         // [2 groups][kStWords][128] states of the rows
+constexpr int kStWords = 14;
+constexpr uint32_t kOffPre = kOffState + kTcGroups * kStWords * kTcRows * 4;  // [2 groups][128] flags of staged rows
+constexpr uint32_t kStageStride = FP_NMOM | 1;                 // floats a staged row (odd: no bank conflicts)
+constexpr uint32_t kOffStage = kOffPre + kTcGroups * kTcRows * 4;  // [128] rows narrowed to FP32 (forming warps)
+constexpr uint32_t kTcSmemUsed = kOffStage + kTcRows * kStageStride * 4;
+static_assert(kTcRows * kStageStride * 4 <= kTcRows * kHid * 2, "the first tiles' rows are staged in A");
+static_assert(kTcRows * 9 * 8 <= kTcRows * kHid * 2, "a tile's coefficients leave through A");
 constexpr size_t kTcSmem = kTcSmemUsed + 1024;                 // room to align the base
 static_assert(kOffBar % 8 == 0, "mbarrier alignment");
 static_assert(kOffScal % 16 == 0, "float4 scalers");
@@ -81,6 +97,19 @@ static_assert(kTcSmem <= 227 * 1024, "shared memory");
 
 __device__ __forceinline__ void group_sync(int g) {
   asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(kTcGroupThreads) : "memory");
+}
+
+// The barriers between group g and the forming warps; each is used in turns
+// (the other side's next arrival follows this side's pass).
+constexpr int kBarFull = 3;     // + g: the tile's inputs and states are in place
+constexpr int kBarXFree = 5;    // + g: the first layer has read the input tile
+constexpr int kBarStFree = 7;   // + g: the output layer has read the states
+constexpr int kBarForm = 9;     // the forming warps among themselves
+__device__ __forceinline__ void pair_sync(int id) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(kTcGroupThreads + kFormThreads) : "memory");
+}
+__device__ __forceinline__ void pair_arrive(int id) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(kTcGroupThreads + kFormThreads) : "memory");
 }
 
 // SiLU(z) = z sigma(z) with sigma(z) = (1 + tanh(z / 2)) / 2: one hardware
@@ -145,16 +174,42 @@ constexpr int kSrcLite = 2;  // LITE inputs from LITE vectors [n][FP_NLITE]
 constexpr int kPreMask = FP_FLAG_FEW | FP_FLAG_SINGULAR | FP_FLAG_NONFINITE;  // the exact closure's preconditions
 constexpr int kFallbackMask = kPreMask | FP_FLAG_RANGE | FP_FLAG_ENERGY;
 
-// what the epilogue of one row needs from its inputs, held by the row's
-// output thread (half 0) from the end of the previous tile to the output
-// layer: the normalised u^_ij, b^_i = u^_ikk and s4^ = w^_kk of the energy
-// check (full inputs), tau, 1 / tau and 1 / (tau sqrt(theta)), and the flags
-// of the inputs this thread formed
+// what the epilogue of one row needs from its inputs: the normalised u^_ij,
+// b^_i = u^_ikk and s4^ = w^_kk of the energy check (full inputs), 1 / tau and
+// 1 / (tau sqrt(theta)), and the flags.  In shared memory one word a row and
+// slot, [kStWords][128] a group: u 0..5, b 6..8, s4 9, itc 10, ig 11, the
+// flags of part 0 (12) and of part 1 (13).
 struct RowState {
   float u[6], b[3], s4, itc, ig;
-  double tc;
   int fl;
 };
+
+template <int kSrc>
+__device__ __forceinline__ void put_state(const RowState &st, float *s) {
+  if constexpr (kSrc == kSrcFull) {
+#pragma unroll
+    for (int a = 0; a < 6; ++a) s[a * kTcRows] = st.u[a];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) s[(6 + a) * kTcRows] = st.b[a];
+    s[9 * kTcRows] = st.s4;
+  }
+  s[10 * kTcRows] = st.itc;
+  s[11 * kTcRows] = st.ig;
+  s[12 * kTcRows] = __int_as_float(st.fl);
+}
+template <int kSrc>
+__device__ __forceinline__ void get_state(RowState &st, const float *s) {
+  if constexpr (kSrc == kSrcFull) {
+#pragma unroll
+    for (int a = 0; a < 6; ++a) st.u[a] = s[a * kTcRows];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) st.b[a] = s[(6 + a) * kTcRows];
+    st.s4 = s[9 * kTcRows];
+  }
+  st.itc = s[10 * kTcRows];
+  st.ig = s[11 * kTcRows];
+  st.fl = __float_as_int(s[12 * kTcRows]) | __float_as_int(s[13 * kTcRows]);
+}
 
 // FP_NMOM or FP_NLITE doubles per row
 template <int kSrc>
@@ -202,71 +257,82 @@ __device__ __forceinline__ int standardise16(const float *f, int q0, int cnt, co
   return fl;
 }
 
-// Inputs of row `row` (cell c) of the next tile, formed by its two threads:
+// The rows [r0, r0 + 128) of the source into shared memory, narrowed to FP32,
+// by kT threads (the forming threads read their rows there: a lane that read
+// its own row from global memory would touch a line a load).  Contiguous
+// 8-byte loads; what FP32 does not show goes to the row's flags: a value that
+// is not finite, a theta that is not positive.
+template <int kSrc, int kT>
+__device__ __forceinline__ void stage_source(const FusedIO &io, int64_t r0, int64_t n, float *stage, int *pre, int t) {
+  constexpr int kS = src_stride<kSrc>(), kPer = kTcRows * kS / kT, kAt = kPer % 15 == 0 ? 15 : 7;  // loads in flight
+  static_assert(kTcRows * kS % kT == 0 && kPer % kAt == 0, "whole rounds");
+  const double *src = io.src + r0 * kS;
+  const int total = (int)(n - r0 < kTcRows ? n - r0 : kTcRows) * kS;
+#pragma unroll 1
+  for (int k0 = 0; k0 < kPer; k0 += kAt) {
+    double x[kAt];
+#pragma unroll
+    for (int k = 0; k < kAt; ++k) {
+      const int i = (k0 + k) * kT + t;
+      x[k] = i < total ? src[i] : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < kAt; ++k) {
+      const int i = (k0 + k) * kT + t, r = i / kS, q = i - r * kS;
+      float f;
+      if (__builtin_expect(!narrow_common(x[k], f) || (q == kTheta && f < 0.f), 0)) {
+        f = narrow(x[k]);
+        if (!finite_d(x[k])) atomicOr(&pre[r], FP_FLAG_NONFINITE);
+        if (q == kTheta && !positive_d(x[k])) atomicOr(&pre[r], FP_FLAG_SINGULAR);
+      }
+      stage[i + r * ((int)kStageStride - kS)] = f;
+    }
+  }
+}
+static_assert(kTheta == 4, "theta's slot in both vectors");
+
+// Inputs of row `row` (cell c) of a tile, formed in two parts from its staged
+// row m (and the flags pre of its staging):
 // part 0 the normalised u_ij / theta and u_ijk / theta^1.5 (features 0..15),
 // the preconditions and the epilogue's state; part 1 w_ij / theta^2 and
 // z_i / theta^2.5 (features 16..24).  Arithmetic as fp_surrogate_features
 // (moments narrowed to FP32, FP32 powers of 1 / theta).
-// Each part writes two 16-byte chunks of the row in X (zeros past n) and its
-// flags (part 0 to `st`, part 1 to `fl_part1`).
-__device__ __forceinline__ void form_full_inputs(const FusedIO &io, const float4 *__restrict__ scal, int64_t c,
-                                                 int64_t n, int part, unsigned char *X, int row, int *fl_part1,
-                                                 RowState &st) {
+// Each part writes two 16-byte chunks of the row in X (zeros past n) and
+// returns its flags.
+__device__ __forceinline__ int form_full_inputs(const FusedIO &io, const float4 *__restrict__ scal, const float *m,
+                                                int pre, int64_t c, int64_t n, int part, unsigned char *X, int row,
+                                                RowState &st) {
   uint32_t pk[8];
   int fl = 0;
   if (c < n) {
-    const double *m = io.src + c * FP_NMOM;
-    const double thd = m[kTheta];
-    const float th = narrow(thd);
+    const float th = m[kTheta];
     const float i1 = 1.f / th;
     const float ih = rsqrtf(th);
     const float i15 = i1 * ih, i2 = i1 * i1, i25 = i2 * ih;
     float f[16];
     if (part == 0) {
-      const double tc = io.tau[c], nd = m[kN];
-      bool fin = finite_d(tc) && positive_d(tc) && finite_d(nd) && finite_d(thd);
+      const double tc = io.tau[c];
+      fl = pre;
+      if (!(finite_d(tc) && positive_d(tc))) fl |= FP_FLAG_NONFINITE;
 #pragma unroll
-      for (int a = 0; a < 6; ++a) {
-        const double v = m[kU2 + a];
-        fin = fin && finite_d(v);
-        f[a] = narrow(v) * i1;
-      }
+      for (int a = 0; a < 6; ++a) f[a] = m[kU2 + a] * i1;
 #pragma unroll
-      for (int a = 0; a < 10; ++a) {
-        const double v = m[kU3 + a];
-        fin = fin && finite_d(v);
-        f[6 + a] = narrow(v) * i15;
-      }
-      if (!fin) fl |= FP_FLAG_NONFINITE;
-      if (narrow(nd) < (float)io.min_particles) fl |= FP_FLAG_FEW;  // N is a whole number
-      if (!positive_d(thd)) fl |= FP_FLAG_SINGULAR;
+      for (int a = 0; a < 10; ++a) f[6 + a] = m[kU3 + a] * i15;
+      if (m[kN] < (float)io.min_particles) fl |= FP_FLAG_FEW;  // N is a whole number
 #pragma unroll
       for (int a = 0; a < 6; ++a) st.u[a] = f[a];
       st.b[0] = f[6 + 0] + f[6 + 3] + f[6 + 5];
       st.b[1] = f[6 + 1] + f[6 + 6] + f[6 + 8];
       st.b[2] = f[6 + 2] + f[6 + 7] + f[6 + 9];
-      st.s4 = narrow(m[kW + 0]) * i2 + narrow(m[kW + 3]) * i2 + narrow(m[kW + 5]) * i2;
+      st.s4 = m[kW + 0] * i2 + m[kW + 3] * i2 + m[kW + 5] * i2;
       st.itc = 1.f / narrow(tc);
       st.ig = st.itc / sqrtf(th);
-      st.tc = tc;
       fl |= standardise16(f, 0, 16, scal, pk);
     } else {
-      bool fin = true;
 #pragma unroll
-      for (int a = 0; a < 3; ++a) fin = fin && finite_d(m[kU + a]);
+      for (int a = 0; a < 6; ++a) f[a] = m[kW + a] * i2;
 #pragma unroll
-      for (int a = 0; a < 6; ++a) {
-        const double v = m[kW + a];
-        fin = fin && finite_d(v);
-        f[a] = narrow(v) * i2;
-      }
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const double v = m[kZ + a];
-        fin = fin && finite_d(v);
-        f[6 + a] = narrow(v) * i25;
-      }
-      if (!fin) fl |= FP_FLAG_NONFINITE;
+      for (int a = 0; a < 3; ++a) f[6 + a] = m[kZ + a] * i25;
       fl |= standardise16(f, 16, kNFeat - 16, scal, pk);
     }
   } else {
@@ -275,35 +341,27 @@ __device__ __forceinline__ void form_full_inputs(const FusedIO &io, const float4
   }
   *reinterpret_cast<uint4 *>(X + cm_off(row, 2 * part, kIn)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
   *reinterpret_cast<uint4 *>(X + cm_off(row, 2 * part + 1, kIn)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-  if (part == 0)
-    st.fl = fl;
-  else
-    *fl_part1 = fl;
+  return fl;
 }
 
-// LITE inputs of row `row` (cell c): both threads form the 16 raw inputs
-// (arithmetic of fp_surrogate_lite_features); part p standardises inputs
-// 8p .. 8p + 7 into chunk p and zeroes chunk 2 + p.
-__device__ __forceinline__ void form_lite_inputs(const FusedIO &io, const float4 *__restrict__ scal, int64_t c,
-                                                 int64_t n, int part, unsigned char *X, int row, int *fl_part1,
-                                                 RowState &st) {
+// LITE inputs of row `row` (cell c) from its staged row m: both parts form
+// the 16 raw inputs (arithmetic of fp_surrogate_lite_features); part p
+// standardises inputs 8p .. 8p + 7 into chunk p and zeroes chunk 2 + p.
+__device__ __forceinline__ int form_lite_inputs(const FusedIO &io, const float4 *__restrict__ scal, const float *m,
+                                                int pre, int64_t c, int64_t n, int part, unsigned char *X, int row,
+                                                RowState &st) {
   uint32_t pk[8];
   int fl = 0;
   if (c < n) {
-    const double *m = io.src + c * FP_NLITE;
     const double tc = io.tau[c];
-    bool fin = finite_d(tc) && positive_d(tc);
-#pragma unroll
-    for (int k = 0; k < FP_NLITE; ++k) fin = fin && finite_d(m[k]);
     float f[16];
     lite_raw_features(m, tc, f);
     if (part == 0) {
-      if (!fin) fl |= FP_FLAG_NONFINITE;
-      if (narrow(m[0]) < (float)io.min_particles) fl |= FP_FLAG_FEW;  // N is a whole number
-      if (!positive_d(m[4])) fl |= FP_FLAG_SINGULAR;
-      st.tc = tc;
+      fl = pre;
+      if (!(finite_d(tc) && positive_d(tc))) fl |= FP_FLAG_NONFINITE;
+      if (m[0] < (float)io.min_particles) fl |= FP_FLAG_FEW;  // N is a whole number
       st.itc = 1.f / narrow(tc);
-      st.ig = st.itc / sqrtf(narrow(m[4]));
+      st.ig = st.itc / sqrtf(m[4]);
       fl |= standardise16(f, 0, 8, scal, pk);
     } else {
       fl |= standardise16(f + 8, 8, 8, scal, pk);
@@ -314,10 +372,16 @@ __device__ __forceinline__ void form_lite_inputs(const FusedIO &io, const float4
   }
   *reinterpret_cast<uint4 *>(X + cm_off(row, part, kIn)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
   *reinterpret_cast<uint4 *>(X + cm_off(row, 2 + part, kIn)) = make_uint4(0u, 0u, 0u, 0u);
-  if (part == 0)
-    st.fl = fl;
+  return fl;
+}
+
+template <int kSrc>
+__device__ __forceinline__ int form_inputs(const FusedIO &io, const float4 *__restrict__ scal, const float *m, int pre,
+                                           int64_t c, int64_t n, int part, unsigned char *X, int row, RowState &st) {
+  if constexpr (kSrc == kSrcFull)
+    return form_full_inputs(io, scal, m, pre, c, n, part, X, row, st);
   else
-    *fl_part1 = fl;
+    return form_lite_inputs(io, scal, m, pre, c, n, part, X, row, st);
 }
 
 // Append cell c to the fallback list when `pick` (warp-aggregated: one
@@ -337,9 +401,13 @@ __device__ __forceinline__ void append_fallback(const FusedIO &io, bool pick, in
 // energy residual e = 1 + (sum_ij C^_ij u^_ij + sum_i G^_i b^_i
 // - eps2_hat s4^) / 3 of the predicted drift is checked and, for a cell that
 // passes every check, C = t / tau and G = t / (tau sqrt(theta)) are scaled in
-// FP32 and widened exactly.  Returns whether the cell goes to the fallback.
+// FP32 and widened exactly into y (shared memory; zeros otherwise, which the
+// fallback overwrites in the caller's array).  Returns whether the cell goes
+// to the fallback.
 __device__ __forceinline__ bool full_epilogue(const FusedIO &io, const float (&v)[kOut], const RowState &st,
-                                              int fl, int64_t c) {
+                                              int fl, int64_t c, double *y) {
+#pragma unroll
+  for (int a = 0; a < 9; ++a) y[a] = 0.0;
   if (!(fl & kPreMask)) {
     bool fin = true;
 #pragma unroll
@@ -350,7 +418,6 @@ __device__ __forceinline__ bool full_epilogue(const FusedIO &io, const float (&v
     if (!fin) fl |= FP_FLAG_NONFINITE;
     if (!(fabsf(e) <= io.energy_tol)) fl |= FP_FLAG_ENERGY;
     if (!(fl & kFallbackMask)) {
-      double *y = io.coeffs + c * 9;
 #pragma unroll
       for (int a = 0; a < 6; ++a) y[a] = f2d_exact(v[a] * st.itc);
 #pragma unroll
@@ -375,14 +442,13 @@ __device__ __forceinline__ void linear_drift(double *y, double tc) {
 // Output epilogue of the LITE closure: degenerate cells and non-finite
 // predictions take the linear drift, the others the scaled predictions.
 __device__ __forceinline__ void lite_epilogue(const FusedIO &io, const float (&v)[kOut], const RowState &st, int fl,
-                                              int64_t c) {
+                                              int64_t c, double *y) {
   bool fin = true;
 #pragma unroll
   for (int a = 0; a < kNOut; ++a) fin = fin && isfinite(v[a]);
   if (!fin) fl |= FP_FLAG_NONFINITE;
-  double *y = io.coeffs + c * 9;
   if (fl & kPreMask) {
-    linear_drift(y, st.tc);
+    linear_drift(y, io.tau[c]);
   } else {
 #pragma unroll
     for (int a = 0; a < 6; ++a) y[a] = f2d_exact(v[a] * st.itc);
@@ -397,10 +463,10 @@ __device__ __forceinline__ void lite_epilogue(const FusedIO &io, const float (&v
 // kSrc = kSrcX: the forward pass on given BF16 inputs x (with kDrop, the
 // dropout masks of the sensitivity probe).  kSrc = kSrcFull / kSrcLite: the
 // learned closure from moment / LITE vectors (io), the inputs formed by the
-// group's threads into the input tile and the coefficients written by the
+// forming warps (the first tiles' by the groups) into the input tile and the coefficients written by the
 // output epilogue; x and out are unused.
 template <bool kDrop, int kSrc>
-__global__ void __launch_bounds__(kTcThreads, 1)
+__global__ void __launch_bounds__(kSrc == kSrcX ? kTcThreads : kTcThreads + kFormThreads, 1)
     mlp_forward_tc_kernel(MlpDev net, const __nv_bfloat16 *__restrict__ x, int64_t n, int standardized_out,
                           float *__restrict__ out, DropoutCfg dc, FusedIO io) {
   static_assert(kSrc == kSrcX || !kDrop, "dropout only on given inputs");
@@ -408,11 +474,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   unsigned char *sm = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   float *bias = reinterpret_cast<float *>(sm + kOffBias);
   float4 *scal = reinterpret_cast<float4 *>(sm + kOffScal);
-  int *fl_part1 = reinterpret_cast<int *>(sm + kOffFlags);
   uint64_t *bar = reinterpret_cast<uint64_t *>(sm + kOffBar);
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sm + kOffTmemSlot);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int g = warp >> 3;                      // group
+  const int g = warp >> 3;                      // group (2: the forming warps)
   const int half = (warp >> 2) & 1;             // which 16 of every 32 columns
   const int row = (warp & 3) * 32 + lane;       // = TMEM lane (warps may use lanes 32 (warp % 4) ..)
 
@@ -421,14 +486,16 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const int64_t tile_step = (int64_t)gridDim.x * kTcGroups;
   int64_t tile = (int64_t)blockIdx.x * kTcGroups + g;
   // the rows of the group's first tile head for L2 while the weights load
-  if (kSrc != kSrcX && tile < n_tiles)
+  if (kSrc != kSrcX && g < kTcGroups && tile < n_tiles)
     prefetch_rows<kSrc>(io, tile * kTcRows, tile * kTcRows + kTcRows < n ? tile * kTcRows + kTcRows : n, gt);
 
   // ---- one-time setup: weights, biases, scalers, barriers, tensor memory ----
-  stage_rows_async(sm + kOffW1, net.W[0], kHid, kIn, kHid, tid, kTcThreads);
-  for (int l = 0; l < 3; ++l)
-    stage_rows_async(sm + kOffWH + l * kHid * kHid * 2, net.W[1 + l], kHid, kHid, kHid, tid, kTcThreads);
-  stage_rows_async(sm + kOffW5, net.W[4], kOut, kHid, kOut, tid, kTcThreads);
+  if (kSrc == kSrcX || g < kTcGroups) {
+    stage_rows_async(sm + kOffW1, net.W[0], kHid, kIn, kHid, tid, kTcThreads);
+    for (int l = 0; l < 3; ++l)
+      stage_rows_async(sm + kOffWH + l * kHid * kHid * 2, net.W[1 + l], kHid, kHid, kHid, tid, kTcThreads);
+    stage_rows_async(sm + kOffW5, net.W[4], kOut, kHid, kOut, tid, kTcThreads);
+  }
   // (the parameter arrays indexed by constants only: no local-memory copy)
   if (tid < kHid) {
 #pragma unroll
@@ -464,22 +531,75 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 
   unsigned char *A = sm + kOffA + g * (kTcRows * kHid * 2);
   unsigned char *X = sm + kOffX + g * (kTcRows * kIn * 2);
-  int *flp = fl_part1 + g * 2 * kTcRows;  // part-1 flags of the group, by tile parity
-  RowState st;
-  // the first tile's inputs while the weight copies land
-  if (tile < n_tiles) {
+  float *state = reinterpret_cast<float *>(sm + kOffState) + g * kStWords * kTcRows;  // the tile's row states
+  // the first tile's inputs while the weight copies land, two threads a row
+  // (the rows staged where the activations go later)
+  if ((kSrc == kSrcX || g < kTcGroups) && tile < n_tiles) {
     if constexpr (kSrc == kSrcX)
       stage_rows_async(X, x + tile * kTcRows * kIn, kTcRows, kIn, n - tile * kTcRows, gt, kTcGroupThreads);
-    else if constexpr (kSrc == kSrcFull)
-      form_full_inputs(io, scal, tile * kTcRows + row, n, half, X, row, flp + row, st);
-    else
-      form_lite_inputs(io, scal, tile * kTcRows + row, n, half, X, row, flp + row, st);
+    else {
+      int *pre = reinterpret_cast<int *>(sm + kOffPre) + g * kTcRows;
+      float *stage = reinterpret_cast<float *>(A);
+      if (half == 0) pre[row] = 0;
+      group_sync(g);
+      stage_source<kSrc, kTcGroupThreads>(io, tile * kTcRows, n, stage, pre, gt);
+      group_sync(g);
+      RowState st;
+      const int fl = form_inputs<kSrc>(io, scal, stage + row * (int)kStageStride, half == 0 ? pre[row] : 0,
+                                       tile * kTcRows + row, n, half, X, row, st);
+      if (half == 0) {
+        st.fl = fl;
+        put_state<kSrc>(st, state + row);
+      } else {
+        state[13 * kTcRows + row] = __int_as_float(fl);
+      }
+    }
   }
   cp_async_wait();
   fence_proxy_async_smem();  // weights written through the generic proxy, read by the MMA
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+
+  // ---- the forming warps (closure variants): every later tile's inputs ----
+  // Two threads a row, for the two groups in turn: the rows are staged while
+  // the group works on its tile, the input tile follows the first layer, the
+  // states the output layer.
+  if (kSrc != kSrcX && g >= kTcGroups) {
+    if constexpr (kSrc != kSrcX) {
+      float *stage = reinterpret_cast<float *>(sm + kOffStage);
+      const int t = tid - kTcThreads, r = t & (kTcRows - 1), part = t / kTcRows;
+      for (int64_t pair = tile_step + (int64_t)blockIdx.x * kTcGroups; pair < n_tiles; pair += tile_step) {
+        for (int q = 0; q < kTcGroups && pair + q < n_tiles; ++q) {
+          const int64_t r0 = (pair + q) * kTcRows;
+          int *pre = reinterpret_cast<int *>(sm + kOffPre) + q * kTcRows;
+          if (part == 0) pre[r] = 0;
+          asm volatile("bar.sync %0, %1;" ::"r"(kBarForm), "r"(kFormThreads) : "memory");
+          stage_source<kSrc, kFormThreads>(io, r0, n, stage, pre, t);
+          const int64_t ahead = r0 + (q + 1 < kTcGroups ? kTcRows : (tile_step - kTcGroups + 1) * kTcRows);
+          if (ahead < n) prefetch_rows<kSrc>(io, ahead, ahead + kTcRows < n ? ahead + kTcRows : n, t);
+          pair_sync(kBarXFree + q);
+          unsigned char *Xq = sm + kOffX + q * (kTcRows * kIn * 2);
+          RowState st;
+          const int fl = form_inputs<kSrc>(io, scal, stage + r * (int)kStageStride, part == 0 ? pre[r] : 0, r0 + r, n,
+                                           part, Xq, r, st);
+          fence_proxy_async_smem();
+          pair_sync(kBarStFree + q);
+          float *sq = reinterpret_cast<float *>(sm + kOffState) + q * kStWords * kTcRows + r;
+          if (part == 0) {
+            st.fl = fl;
+            put_state<kSrc>(st, sq);
+          } else {
+            sq[13 * kTcRows] = __int_as_float(fl);
+          }
+          pair_arrive(kBarFull + q);
+        }
+      }
+    }
+    __syncthreads();  // the teardown's
+    return;
+  }
+
   const uint32_t tmem = *tmem_slot + (uint32_t)(g * 2 * kHid);  // the group's two accumulators
   const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;   // this warp's TMEM lanes
   const uint32_t a_addr = smem_u32(A), x_addr = smem_u32(X);
@@ -501,22 +621,25 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   for (int it = 0; tile < n_tiles; tile += tile_step, ++it) {
     const int64_t row0 = tile * kTcRows;
     const int64_t next = tile + tile_step;
+    double *yt = reinterpret_cast<double *>(A);  // the tile's coefficients on their way out
+    bool x_freed = false;
+    if constexpr (kSrc == kSrcX) {
+      cp_async_wait();  // this thread's part of the input tile has landed
+      fence_proxy_async_smem();
+    }
+    tc_fence_before();
+    if (kSrc != kSrcX && it > 0)
+      pair_sync(kBarFull + g);
+    else
+      group_sync(g);
     if (!failed) {
       // layer 1: D[0] = X W1^T
-      if constexpr (kSrc == kSrcX) cp_async_wait();  // this thread's part of the input tile has landed
-      fence_proxy_async_smem();
-      tc_fence_before();
-      group_sync(g);
       if (leader) {
         tc_fence_after();
         for (int s = 0; s < kIn / 16; ++s)
           tc_mma(tmem, smem_desc(x_addr + 256 * s, 128, kIn * 16), smem_desc(w1_addr + 256 * s, 128, kIn * 16),
                  idesc_bf16(kTcRows, kHid), s > 0 ? 1u : 0u);
         tc_commit(&bar[g]);
-      }
-      if (kSrc != kSrcX && next < n_tiles) {
-        const int64_t r1 = next * kTcRows + kTcRows < n ? next * kTcRows + kTcRows : n;
-        prefetch_rows<kSrc>(io, next * kTcRows, r1, gt);
       }
       // hidden layers l = 0..3: epilogue of D[l & 1], MMAs of layer l + 1
 #pragma unroll 1
@@ -525,9 +648,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           failed = true;
           break;
         }
-        if constexpr (kSrc == kSrcX)
-          if (l == 0 && next < n_tiles)  // X is free: stage the next input tile
+        if (l == 0 && next < n_tiles) {  // X is free: the next input tile
+          if constexpr (kSrc == kSrcX)
             stage_rows_async(X, x + next * kTcRows * kIn, kTcRows, kIn, n - next * kTcRows, gt, kTcGroupThreads);
+          else
+            pair_arrive(kBarXFree + g);
+          x_freed = true;
+        }
         const uint32_t d_in = tmem + (uint32_t)((l & 1) * kHid), d_out = tmem + (uint32_t)(((l + 1) & 1) * kHid);
         const int n_next = l == 3 ? kOut : kHid;
         const uint32_t w_next = l == 3 ? w5_addr : wh_addr + (uint32_t)(l * kHid * kHid * 2);
@@ -580,11 +707,22 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             for (int q = 0; q < kOut / 2; ++q) o[q] = make_float2(v[2 * q], v[2 * q + 1]);
           }
         } else if constexpr (kSrc == kSrcFull) {
-          const bool pick = c < n && full_epilogue(io, v, st, st.fl | flp[(it & 1) * kTcRows + row], c);
+          RowState st;
+          get_state<kSrc>(st, state + row);
+          const bool pick = c < n && full_epilogue(io, v, st, st.fl, c, yt + row * 9);
           append_fallback(io, pick, c, lane);
         } else {
-          if (c < n) lite_epilogue(io, v, st, st.fl | flp[(it & 1) * kTcRows + row], c);
+          RowState st;
+          get_state<kSrc>(st, state + row);
+          if (c < n) lite_epilogue(io, v, st, st.fl, c, yt + row * 9);
         }
+      }
+      if (kSrc != kSrcX && !failed) {
+        // the tile's coefficients, contiguous, by the whole group (its
+        // activations are free: the output layer has read them)
+        group_sync(g);
+        const int total = (int)(n - row0 < kTcRows ? n - row0 : kTcRows) * 9;
+        for (int i = gt; i < total; i += kTcGroupThreads) io.coeffs[row0 * 9 + i] = yt[i];
       }
     }
     if (failed) {
@@ -611,13 +749,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           }
         }
       }
-    } else if (kSrc != kSrcX && next < n_tiles) {
-      // the next tile's inputs: X is free since the first layer's MMAs of
-      // this tile completed; part-1 flags go to the other parity slot
-      if constexpr (kSrc == kSrcFull)
-        form_full_inputs(io, scal, next * kTcRows + row, n, half, X, row, flp + ((it + 1) & 1) * kTcRows + row, st);
-      else if constexpr (kSrc == kSrcLite)
-        form_lite_inputs(io, scal, next * kTcRows + row, n, half, X, row, flp + ((it + 1) & 1) * kTcRows + row, st);
+    }
+    if (kSrc != kSrcX && next < n_tiles) {
+      if (!x_freed) pair_arrive(kBarXFree + g);
+      pair_arrive(kBarStFree + g);
     }
   }
   // ---- teardown ----
@@ -666,8 +801,9 @@ static int launch_tc(const MlpDev &net, const __nv_bfloat16 *x, int64_t n, int s
   int64_t grid = (n_tiles + kTcGroups - 1) / kTcGroups;
   if (grid > tc_sm_count()) grid = tc_sm_count();
   if (grid < 1) grid = 1;
-  mlp_forward_tc_kernel<kDrop, kSrc><<<(unsigned)grid, kTcThreads, kTcSmem, st>>>(net, x, n, standardized_out, out,
-                                                                                   dc, io);
+  constexpr int threads = kSrc == kSrcX ? kTcThreads : kTcThreads + kFormThreads;
+  mlp_forward_tc_kernel<kDrop, kSrc><<<(unsigned)grid, threads, kTcSmem, st>>>(net, x, n, standardized_out, out, dc,
+                                                                               io);
   return 0;
 }
 

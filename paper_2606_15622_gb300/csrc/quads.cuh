@@ -108,8 +108,7 @@ __device__ __forceinline__ float narrow<float>(double x) {
 // row l at stage + l (NK | 1) (an odd stride: the lanes then read their own
 // rows without bank conflicts).  The warp's loads are contiguous; a lane that
 // read its own row from global memory would touch a line a load (32 wavefronts
-// an instruction).  The narrowing stays on the FP64 pipe, which these kernels
-// leave idle (d2f_rn's integers: 100 us against 83 for the adjoint's pass).
+// an instruction).
 // `more` (if not null): a second set of rows, loaded beside the first into
 // stage + more_at.
 template <int NK, typename T>
