@@ -55,16 +55,16 @@ __host__ __device__ __forceinline__ void assembly_vjp(const double (&m)[FP_NMOM]
 #pragma unroll
   for (int i = 0; i < 3; ++i) b[i] = m[kU3 + sym3(i, 0, 0)] + m[kU3 + sym3(i, 1, 1)] + m[kU3 + sym3(i, 2, 2)];
   const double th = m[kTheta];
-  const double itau = 1.0 / tc, ith = 1.0 / th;
+  const double itau = rcp_d(tc), ith = rcp_d(th);
   const double e2 = eps2_hat * itau * ith;
   // per-cell factors of the row adjoints
-  const double itau2 = 2.0 * itau, me2x2 = -2.0 * e2, e2x2 = 2.0 * e2, mz = -3.0 * e2;
+  const double itau2 = times_pow2<1>(itau), e2x2 = times_pow2<1>(e2), me2x2 = -e2x2, mz = -3.0 * e2;
   const double kb = fma(4.0 / 3.0, itau, 3.0 * e2 * th);  // heat row i on b_i
   const double m18th = -18.0 * th, m6th = -6.0 * th, e2x3 = 3.0 * e2, th3 = 3.0 * th;
   double G2[3], G6[3], eb2[3], P[3], E[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    G2[k] = 2.0 * G[k];
+    G2[k] = times_pow2<1>(G[k]);
     G6[k] = m6th * G[k];
     eb2[k] = e2x2 * b[k];
   }
@@ -85,13 +85,20 @@ __host__ __device__ __forceinline__ void assembly_vjp(const double (&m)[FP_NMOM]
 #pragma unroll
     for (int j = i; j < 3; ++j) {
       const double f = -lam[sym2(i, j)];
+      if (i == j) {  // the two terms of each sum are the same
+        const double f2 = times_pow2<1>(f);
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        ub[k][j] = fma(f, C[i][k], ub[k][j]);
-        ub[k][i] = fma(f, C[j][k], ub[k][i]);
+        for (int k = 0; k < 3; ++k) ub[k][i] = fma(f2, C[i][k], ub[k][i]);
+        bb[i] = fma(f2, G[i], bb[i]);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          ub[k][j] = fma(f, C[i][k], ub[k][j]);
+          ub[k][i] = fma(f, C[j][k], ub[k][i]);
+        }
+        bb[j] = fma(f, G[i], bb[j]);
+        bb[i] = fma(f, G[j], bb[i]);
       }
-      bb[j] = fma(f, G[i], bb[j]);
-      bb[i] = fma(f, G[j], bb[i]);
       ub[i][j] = fma(f, itau2, ub[i][j]);
       wb[i][j] = fma(f, me2x2, wb[i][j]);
       sw = fma(f, w[i][j], sw);  // e2 adjoint: -2 sum f w_ij
@@ -99,7 +106,7 @@ __host__ __device__ __forceinline__ void assembly_vjp(const double (&m)[FP_NMOM]
   // heat-flux rows
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    const double f = -lam[6 + i], f2 = 2.0 * f, f4 = 4.0 * f, fe = e2x2 * f;
+    const double f = -lam[6 + i], f2 = times_pow2<1>(f), f4 = times_pow2<2>(f), fe = e2x2 * f;
 #pragma unroll
     for (int l = 0; l < 3; ++l) bb[l] = fma(f, C[i][l], bb[l]);
     // 2 sum_kl C_kl u_ikl: a slot with k != l collects (k, l) and (l, k)
@@ -185,7 +192,9 @@ __device__ __forceinline__ void adjoint_cell(int64_t c, const double *__restrict
         for (int j = 0; j < 9; ++j) at[i][j] = a[j][i];
         at[i][9] = gY[c * 9 + i];
       }
-      pivoted_solve(at, 0.0, lam);
+      double rinv[9];
+      uint64_t perm;
+      pivoted_solve<false, true>(at, 0.0, lam, rinv, perm);
     }
     double Y[9];
 #pragma unroll
@@ -199,12 +208,14 @@ __device__ __forceinline__ void adjoint_cell(int64_t c, const double *__restrict
   for (int k = 0; k < FP_NMOM; ++k) gm_out[c * FP_NMOM + k] = gm[k];
 }
 
-// One thread per cell, grid-stride, two 128-thread blocks per SM (FP64-bound:
-// see solve_kernel), registers capped at 128 a thread (the rest spills to
-// L1): half the register file stays free for the velocity update and the
-// learned closure running beside it.
+// One thread per cell, grid-stride, FP64-bound (see solve_kernel; 306
+// instructions a cell with the factors, 72 us of 131,072 cells).  With the
+// factors three 128-thread blocks per SM, for the loads of the factors: 82 us,
+// 89 with two capped at 128 registers and the FP64 reciprocals, 90 with four
+// today.  Without them two blocks and no cap: 16,384 cells 29.8 us, 33 with
+// the cap.
 template <bool kLU>
-__global__ void __launch_bounds__(128, 4) adjoint_cell_kernel(const double *__restrict__ mom,
+__global__ void __launch_bounds__(128, kLU ? 3 : 2) adjoint_cell_kernel(const double *__restrict__ mom,
                                                               const double *__restrict__ coeffs,
                                                               const int32_t *__restrict__ flags,
                                                               const double *__restrict__ lu,
@@ -704,8 +715,9 @@ void launch_adjoint(const void *v, int v_dtype, int64_t np, const int64_t *off, 
                     const double *gY, const double *gm_in, double *gm_out, void *gv, cudaStream_t st) {
   {
     const int threads = 128;
+    const int per_sm = lu ? 3 : 2;
     int64_t blocks = (n_cells + threads - 1) / threads;
-    if (blocks > 2 * adj_sm_count()) blocks = 2 * adj_sm_count();
+    if (blocks > per_sm * adj_sm_count()) blocks = per_sm * adj_sm_count();
     if (lu)
       adjoint_cell_kernel<true><<<(unsigned)blocks, threads, 0, st>>>(mom, coeffs, flags, lu, tau, gY, gm_in,
                                                                       n_cells, eps2_hat, gm_out);

@@ -197,13 +197,17 @@ __global__ void __launch_bounds__(256) gather_fp32_kernel(const VT *__restrict__
 // ---------------------------------------------------------------------------
 // One thread per cell, grid-stride over two resident 128-thread blocks per SM;
 // two warps per SM sub-partition keep its FP64 unit busy through each
-// other's dependency stalls.  The registers are capped at 168 a thread (some
-// of the 9 x 10 system spills to L1): alone the kernel is as fast as with
-// the whole register file, and the third of the file it leaves free lets the
-// learned closure's kernels run beside it in the step.  With kLU the factors
-// of P A = L U of every unflagged cell go to lu for the adjoint.
+// other's dependency stalls.  Bound by the FP64 instructions, 392 a cell at 68
+// cycles a warp: 131,072 cells 102 us, with the factors stored 110; 150 and
+// 158 with divisions for the reciprocals, products by two and four, the
+// structurally zero rows and |a| compared on the FP64 pipe (511 and more).
+// Without the factors the registers are capped at 168 a thread (some of the 9
+// x 10 system spills to L1; uncapped 99 us): the third of the file left free
+// lets the learned closure's kernels run beside it in the step.  With kLU the
+// factors of P A = L U of every unflagged cell go to lu for the adjoint
+// (capped 116).
 template <bool kLU>
-__global__ void __launch_bounds__(128, 3) solve_kernel(const double *__restrict__ mom, const double *__restrict__ tau,
+__global__ void __launch_bounds__(128, kLU ? 2 : 3) solve_kernel(const double *__restrict__ mom, const double *__restrict__ tau,
                                                        int64_t n_cells, SolveParams prm, double *__restrict__ coeffs,
                                                        int32_t *__restrict__ flags, double *__restrict__ lu) {
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n_cells;
@@ -355,7 +359,7 @@ void launch_solve(const double *mom, const double *tau, int64_t n_cells, const f
   const unsigned three = (unsigned)(blocks < 3 * sm_count() ? blocks : 3 * sm_count());
   // a half warp a cell while every SM sub-partition has one warp of them at
   // most (eight times the FP64 instructions a cell, half the chain): 400 cells
-  // 16.5 us against 25.3
+  // 13.4 us against 21
   const bool few = n_cells <= 8 * (int64_t)sm_count();
   if (lu)
     solve_kernel<true><<<two, threads, 0, st>>>(mom, tau, n_cells, prm, coeffs, flags, lu);

@@ -29,6 +29,21 @@ static_assert(sym3(2, 0, 1) == 4 && sym3(1, 2, 2) == 8 && sym3(2, 1, 1) == 7 && 
 __device__ __forceinline__ double tfma(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float tfma(float a, float b, float c) { return fmaf(a, b, c); }
 
+// times 2 or 4, reciprocals and quotients: in FP64 without the FP64 pipe or
+// with three of its instructions
+template <int k>
+__device__ __forceinline__ double tpow2(double a) { return times_pow2<k>(a); }
+template <int k>
+__device__ __forceinline__ float tpow2(float a) { return (float)(1 << k) * a; }
+// a b + c: in FP64 one rounding by its spelling (the kernels that share these
+// expressions give the same bits), in FP32 as the compiler contracts it
+__device__ __forceinline__ double tmad(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float tmad(float a, float b, float c) { return a * b + c; }
+__device__ __forceinline__ double trcp(double a) { return rcp_d(a); }
+__device__ __forceinline__ float trcp(float a) { return 1.f / a; }
+__device__ __forceinline__ double tquot(double a, double b) { return a * rcp_d(b); }
+__device__ __forceinline__ float tquot(float a, float b) { return a / b; }
+
 struct SolveParams {
   double eps2_hat;
   double pivot_rtol;
@@ -63,9 +78,9 @@ __device__ __forceinline__ void assemble_emit(const T (&m)[FP_NMOM], T tau, T ep
     b[i] = m[kU3 + sym3(i, 0, 0)] + m[kU3 + sym3(i, 1, 1)] + m[kU3 + sym3(i, 2, 2)];
   const T theta = m[kTheta];
   const T s4 = w[0][0] + w[1][1] + w[2][2];
-  const T eps2 = eps2_hat / (tau * theta);
-  const T inv_tau = T(1) / tau;
-  const T c_u = T(-2) * inv_tau, c_w = T(2) * eps2;  // stress right-hand side
+  const T eps2 = tquot(eps2_hat, tau * theta);
+  const T inv_tau = trcp(tau);
+  const T c_u = -tpow2<1>(inv_tau), c_w = tpow2<1>(eps2);  // stress right-hand side
   const T th3 = T(3) * theta;
   // stress rows
 #pragma unroll
@@ -76,8 +91,8 @@ __device__ __forceinline__ void assemble_emit(const T (&m)[FP_NMOM], T tau, T ep
       if (i == j) {
         // 2 sum_k C_ik u_ki + 2 G_i b_i
 #pragma unroll
-        for (int k = 0; k < 3; ++k) emit(row, sym2(i, k), T(2) * u[k][i]);
-        emit(row, 6 + i, T(2) * b[i]);
+        for (int k = 0; k < 3; ++k) emit(row, sym2(i, k), tpow2<1>(u[k][i]));
+        emit(row, 6 + i, tpow2<1>(b[i]));
       } else {
         // C_ii u_ij + C_jj u_ij + C_ij (u_ii + u_jj) + C_it u_tj + C_jt u_ti
         const int t = 3 - i - j;
@@ -89,7 +104,7 @@ __device__ __forceinline__ void assemble_emit(const T (&m)[FP_NMOM], T tau, T ep
         emit(row, 6 + i, b[j]);
         emit(row, 6 + j, b[i]);
       }
-      emit(row, 9, c_u * u[i][j] + c_w * w[i][j]);
+      emit(row, 9, tmad(c_u, u[i][j], c_w * w[i][j]));
     }
   // heat-flux rows
 #pragma unroll
@@ -111,15 +126,16 @@ __device__ __forceinline__ void assemble_emit(const T (&m)[FP_NMOM], T tau, T ep
           has_b = true;
         }
         const T f = p == q ? T(2) : T(4);
-        emit(row, sym2(p, q), has_b ? tfma(f, u3, bterm) : f * u3);
+        emit(row, sym2(p, q), has_b ? tfma(f, u3, bterm) : (p == q ? tpow2<1>(u3) : tpow2<2>(u3)));
       }
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const T gk = T(2) * tfma(-th3, u[k][i], w[k][i]);
-      emit(row, 6 + k, k == i ? (s4 - T(9) * theta * theta) + gk : gk);
+      const T gk = tpow2<1>(tfma(-th3, u[k][i], w[k][i]));
+      emit(row, 6 + k, k == i ? tmad(T(-9) * theta, theta, s4) + gk : gk);
     }
-    const T ub = u[i][0] * b[0] + u[i][1] * b[1] + u[i][2] * b[2];
-    emit(row, 9, T(-4.0 / 3.0) * inv_tau * b[i] + eps2 * (T(3) * m[kZ + i] - th3 * b[i] - T(2) * ub));
+    const T ub = tmad(u[i][2], b[2], tmad(u[i][1], b[1], u[i][0] * b[0]));
+    const T q = tmad(T(-2), ub, tmad(-th3, b[i], T(3) * m[kZ + i]));
+    emit(row, 9, tmad(eps2, q, T(-4.0 / 3.0) * inv_tau * b[i]));
   }
 }
 
@@ -132,18 +148,30 @@ __device__ __forceinline__ void assemble(const double (&m)[FP_NMOM], double tau,
   assemble_emit(m, tau, eps2_hat, [&](int row, int col, double v) { a[row][col] = v; });
 }
 
+// Whether row i of A (of A^T with kT) is zero in column K whatever the
+// moments, before and after the earlier steps: C_11 is in none of the rows 22,
+// 23 and 33, C_12 not in the row 33; the row 11 holds no C_22, C_23, C_33, G_2
+// or G_3, the row 12 no C_33 and no G_3 (rows that step 0 leaves alone).  39 of
+// the elimination's 276 multiply-adds and products, 68 of the transposed one's.
+__host__ __device__ constexpr bool skip_row(int K, int i, bool kT) {
+  return K == 0 ? (i >= 3 && i <= 5) || (kT && i >= 7) : K == 1 && (i == 5 || (kT && i == 8));
+}
+
 // One elimination step for column K (a template so every index is static and
 // the matrix stays in registers).  With kLU the whole rows are swapped and
 // the multipliers are kept below the diagonal, so that afterwards P A = L U
 // with L unit lower triangular in a[i][j < i], U in a[i][j >= i], and the
-// row swapped with row K at step K in bits 4K..4K+3 of perm.
-template <int K, bool kLU>
+// row swapped with row K at step K in bits 4K..4K+3 of perm.  Rows that are
+// zero in column K by the system's structure (skip_row) are neither candidates
+// nor changed.
+template <int K, bool kLU, bool kT>
 __device__ __forceinline__ void elim_step(double (&a)[9][10], uint64_t thr, int &flag, double (&rinv)[9],
                                           uint64_t &perm) {
   uint64_t best = abs_bits(a[K][K]);
   int bi = K;
 #pragma unroll
   for (int i = K + 1; i < 9; ++i) {
+    if (skip_row(K, i, kT)) continue;
     const uint64_t bb = abs_bits(a[i][K]);
     if (bb > best) {
       best = bb;
@@ -154,6 +182,7 @@ __device__ __forceinline__ void elim_step(double (&a)[9][10], uint64_t thr, int 
   if (kLU) perm |= (uint64_t)bi << (4 * K);
 #pragma unroll
   for (int i = K + 1; i < 9; ++i) {
+    if (skip_row(K, i, kT)) continue;
     const bool sw = (bi == i);
 #pragma unroll
     for (int j = kLU ? 0 : K; j < 10; ++j) {
@@ -162,9 +191,10 @@ __device__ __forceinline__ void elim_step(double (&a)[9][10], uint64_t thr, int 
       a[i][j] = sw ? t : a[i][j];
     }
   }
-  rinv[K] = 1.0 / a[K][K];
+  rinv[K] = rcp_d(a[K][K]);
 #pragma unroll
   for (int i = K + 1; i < 9; ++i) {
+    if (skip_row(K, i, kT)) continue;
     const double l = a[i][K] * rinv[K];
     if (kLU) a[i][K] = l;
 #pragma unroll
@@ -173,10 +203,11 @@ __device__ __forceinline__ void elim_step(double (&a)[9][10], uint64_t thr, int 
 }
 
 // Partial-pivot elimination and back substitution on [A | r]; returns
-// FP_FLAG_SINGULAR if a pivot is <= rtol * max|A| (y is then garbage).
+// FP_FLAG_SINGULAR if a pivot is <= rtol * max|A| (y is then garbage).  a
+// holds an assembled system, with kT its transpose.
 // With kLU the factors stay in a (see elim_step), rinv holds the reciprocal
 // pivots and perm the row swaps.
-template <bool kLU = false>
+template <bool kLU = false, bool kT = false>
 __device__ __forceinline__ int pivoted_solve(double (&a)[9][10], double rtol, double (&y)[9], double (&rinv)[9],
                                              uint64_t &perm) {
   uint64_t amax = 0;
@@ -189,15 +220,15 @@ __device__ __forceinline__ int pivoted_solve(double (&a)[9][10], double rtol, do
   if (!(amax_d > 0.0) || !finite_d(amax_d)) flag = FP_FLAG_SINGULAR;
   const uint64_t thr = abs_bits(rtol * amax_d);
   perm = 0;
-  elim_step<0, kLU>(a, thr, flag, rinv, perm);
-  elim_step<1, kLU>(a, thr, flag, rinv, perm);
-  elim_step<2, kLU>(a, thr, flag, rinv, perm);
-  elim_step<3, kLU>(a, thr, flag, rinv, perm);
-  elim_step<4, kLU>(a, thr, flag, rinv, perm);
-  elim_step<5, kLU>(a, thr, flag, rinv, perm);
-  elim_step<6, kLU>(a, thr, flag, rinv, perm);
-  elim_step<7, kLU>(a, thr, flag, rinv, perm);
-  elim_step<8, kLU>(a, thr, flag, rinv, perm);
+  elim_step<0, kLU, kT>(a, thr, flag, rinv, perm);
+  elim_step<1, kLU, kT>(a, thr, flag, rinv, perm);
+  elim_step<2, kLU, kT>(a, thr, flag, rinv, perm);
+  elim_step<3, kLU, kT>(a, thr, flag, rinv, perm);
+  elim_step<4, kLU, kT>(a, thr, flag, rinv, perm);
+  elim_step<5, kLU, kT>(a, thr, flag, rinv, perm);
+  elim_step<6, kLU, kT>(a, thr, flag, rinv, perm);
+  elim_step<7, kLU, kT>(a, thr, flag, rinv, perm);
+  elim_step<8, kLU, kT>(a, thr, flag, rinv, perm);
 #pragma unroll
   for (int k = 8; k >= 0; --k) {
     double s = a[k][9];
@@ -206,11 +237,6 @@ __device__ __forceinline__ int pivoted_solve(double (&a)[9][10], double rtol, do
     y[k] = s * rinv[k];
   }
   return flag;
-}
-__device__ __forceinline__ int pivoted_solve(double (&a)[9][10], double rtol, double (&y)[9]) {
-  double rinv[9];
-  uint64_t perm;
-  return pivoted_solve<false>(a, rtol, y, rinv, perm);
 }
 
 // Stored factors: FP_LU_STRIDE doubles per cell -- L below / reciprocal
@@ -268,12 +294,12 @@ __device__ __forceinline__ int closure_cell(const double *__restrict__ mc, doubl
 #pragma unroll
   for (int k = 0; k < FP_NMOM; ++k) m[k] = mc[k];
   int fl = 0;
-  bool fin = finite_d(tc) && tc > 0.0;
+  bool fin = finite_d(tc) && positive_d(tc);
 #pragma unroll
   for (int k = 0; k < FP_NMOM; ++k) fin = fin && finite_d(m[k]);
   if (!fin) fl |= FP_FLAG_NONFINITE;
   if (m[kN] < (double)prm.min_particles) fl |= FP_FLAG_FEW;
-  if (!(m[kTheta] > 0.0)) fl |= FP_FLAG_SINGULAR;
+  if (!positive_d(m[kTheta])) fl |= FP_FLAG_SINGULAR;
   if (!fl && m[kN] < (double)prm.min_regular) fl |= FP_FLAG_SINGULAR;
   if (!fl) {
     double a[9][10], rinv[9];
@@ -462,6 +488,7 @@ __device__ __forceinline__ void lu_step_f(float (&a)[9][10], float (&rinv)[9], u
   int bi = K;
 #pragma unroll
   for (int i = K + 1; i < 9; ++i) {
+    if (skip_row(K, i, false)) continue;
     const uint32_t bb = __float_as_uint(a[i][K]) & 0x7fffffffu;
     if (bb > best) {
       best = bb;
@@ -472,6 +499,7 @@ __device__ __forceinline__ void lu_step_f(float (&a)[9][10], float (&rinv)[9], u
   perm |= (uint64_t)bi << (4 * K);
 #pragma unroll
   for (int i = K + 1; i < 9; ++i) {
+    if (skip_row(K, i, false)) continue;
     const bool sw = (bi == i);
 #pragma unroll
     for (int j = 0; j < 10; ++j) {
@@ -483,6 +511,7 @@ __device__ __forceinline__ void lu_step_f(float (&a)[9][10], float (&rinv)[9], u
   rinv[K] = 1.f / a[K][K];
 #pragma unroll
   for (int i = K + 1; i < 9; ++i) {
+    if (skip_row(K, i, false)) continue;
     const float l = a[i][K] * rinv[K];
     a[i][K] = l;
 #pragma unroll
@@ -550,7 +579,7 @@ __device__ __forceinline__ int closure_cell_mixed(const double *__restrict__ mc,
   int fl = 0;
   bool in_range;  // of f2_split: theta and tau within 2^+-20, so z (order 5) within 2^+-50 of one
   {
-    bool fin = finite_d(tc) && tc > 0.0;
+    bool fin = finite_d(tc) && positive_d(tc);
 #pragma unroll
     for (int k = 0; k < FP_NMOM; ++k) fin = fin && finite_d(mc[k]);
     if (!fin) fl |= FP_FLAG_NONFINITE;
@@ -625,9 +654,9 @@ __device__ __forceinline__ int closure_cell_mixed(const double *__restrict__ mc,
 // a_iK * (1 / a_KK), fma updates, the sum over j ascending), so coefficients
 // and flags are identical; what changes is the length of the dependent chain
 // (FP64 instructions have a latency of about 64 cycles on this GPU, a
-// division about 550), roughly halved, which is what a short fallback list
-// waits for.  The division by each candidate pivot runs beside the pivot
-// search.  The solve runs even for a flagged cell (the warp must stay
+// reciprocal by rcp_d about 400), roughly halved, which is what a short
+// fallback list waits for.  The reciprocal of each candidate pivot runs beside
+// the pivot search.  The solve runs even for a flagged cell (the warp must stay
 // converged for the shuffles) and its result is then discarded; valid =
 // false makes the group a passenger: no loads, results meaningless.
 __device__ __forceinline__ int closure_cell_group16(const double *__restrict__ mc, double tc, const SolveParams &prm,
@@ -637,12 +666,12 @@ __device__ __forceinline__ int closure_cell_group16(const double *__restrict__ m
 #pragma unroll
   for (int k = 0; k < FP_NMOM; ++k) m[k] = valid ? mc[k] : 1.0;
   int fl = 0;
-  bool fin = finite_d(tc) && tc > 0.0;
+  bool fin = finite_d(tc) && positive_d(tc);
 #pragma unroll
   for (int k = 0; k < FP_NMOM; ++k) fin = fin && finite_d(m[k]);
   if (!fin) fl |= FP_FLAG_NONFINITE;
   if (m[kN] < (double)prm.min_particles) fl |= FP_FLAG_FEW;
-  if (!(m[kTheta] > 0.0)) fl |= FP_FLAG_SINGULAR;
+  if (!positive_d(m[kTheta])) fl |= FP_FLAG_SINGULAR;
   if (!fl && m[kN] < (double)prm.min_regular) fl |= FP_FLAG_SINGULAR;
 
   double row[10];
@@ -664,7 +693,7 @@ __device__ __forceinline__ int closure_cell_group16(const double *__restrict__ m
   double rinv[9];
 #pragma unroll
   for (int K = 0; K < 9; ++K) {
-    const double inv_own = 1.0 / row[K];  // this lane's candidate reciprocal, beside the search
+    const double inv_own = rcp_d(row[K]);  // this lane's candidate reciprocal, beside the search
     // pivot: the largest |a_iK| over rows i >= K, the first such row on ties
     // (key 0 for lanes that are not candidates)
     const bool cand = r >= K && r < 9;

@@ -74,11 +74,94 @@ __device__ __forceinline__ double u2d_exact(uint32_t n) {
   return __longlong_as_double((long long)(((uint64_t)(e + 1023) << 52) | frac));
 }
 
+// |x| as its bits, put together from the halves: masked as one 64-bit word the
+// compiler sees an absolute value and takes it, and the comparisons, to the
+// FP64 pipe
 __device__ __forceinline__ uint64_t abs_bits(double x) {
-  return (uint64_t)__double_as_longlong(x) & 0x7fffffffffffffffull;
+  uint32_t hi = (uint32_t)__double2hiint(x) & 0x7fffffffu;
+  asm("" : "+r"(hi));
+  return ((uint64_t)hi << 32) | (uint32_t)__double2loint(x);
 }
 __device__ __forceinline__ bool finite_d(double x) {
   return (abs_bits(x) & 0x7ff0000000000000ull) != 0x7ff0000000000000ull;
+}
+
+// x 2^k exactly on the integer pipe: the exponent's field raised, a subnormal
+// shifted (its leading bit moves into the exponent), an overflow to infinity,
+// infinities and NaN as they are.
+template <int k>
+__host__ __device__ __forceinline__ double times_pow2(double x) {
+#ifdef __CUDA_ARCH__
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t a = hi & 0x7fffffffu;
+  uint32_t h = hi + ((uint32_t)k << 20), l = lo;
+  if (__builtin_expect(a - (1u << 20) >= (uint32_t)(2046 - k) << 20, 0)) {
+    asm volatile("" : "+r"(l));  // a branch, not computed beside the common case
+    uint64_t b = ((uint64_t)a << 32) | lo;
+#pragma unroll
+    for (int i = 0; i < k; ++i) {
+      if (b < (1ull << 52))
+        b <<= 1;
+      else if (b < (2047ull << 52))
+        b = b >= (2046ull << 52) ? 2047ull << 52 : b + (1ull << 52);
+    }
+    h = (uint32_t)(b >> 32) | (hi & 0x80000000u);
+    l = (uint32_t)b;
+  }
+  return __hiloint2double((int)h, (int)l);
+#else
+  return x * (double)(1 << k);
+#endif
+}
+
+// 1 / p from the hardware's FP32 reciprocal of p's mantissa (good to about
+// 2^-22) and one step of third order on it, x (1 + e + e^2) with e = 1 - m x:
+// what is left out, e^3, is below 2^-64, so the result is within a little over
+// half a unit in the last place (a subnormal one is cut off).  The exponent and
+// the special values are put in by integer operations: three FP64 instructions
+// where the division takes about ten.
+__host__ __device__ __forceinline__ double rcp_d(double p) {
+#ifdef __CUDA_ARCH__
+  const uint32_t hi = (uint32_t)__double2hiint(p), sign = hi & 0x80000000u;
+  uint32_t mh = hi & 0x000fffffu, ml = (uint32_t)__double2loint(p);  // the fraction
+  int ex = (int)((hi >> 20) & 0x7ffu);
+  if (__builtin_expect(ex == 0, 0)) {  // subnormal: the leading bit to the place before the fraction
+    asm volatile("" : "+r"(mh));       // (a branch, as below)
+    const uint64_t f = ((uint64_t)mh << 32) | ml;
+    const int sh = f ? __clzll((long long)f) - 11 : 0;
+    mh = (uint32_t)((f << sh) >> 32) & 0x000fffffu;
+    ml = (uint32_t)(f << sh);
+    ex = f ? 1 - sh : -2000;  // (zero: infinity below)
+  }
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(0x3f800000u | __funnelshift_l(ml, mh, 3))));
+  const uint32_t rb = __float_as_uint(r);  // in [1/2, 1]
+  const double m = __hiloint2double((int)(mh | 0x3ff00000u), (int)ml);
+  double x = __hiloint2double((int)((rb >> 3) + (896u << 20)), (int)(rb << 29));
+  double e = fma(-m, x, 1.0);
+  e = fma(e, e, e);
+  x = fma(x, e, x);
+  const uint32_t xh = (uint32_t)__double2hiint(x);
+  uint32_t oh = xh + ((uint32_t)(1023 - ex) << 20), ol = (uint32_t)__double2loint(x);
+  if (__builtin_expect((unsigned)(ex - 1) >= 2044u, 0)) {
+    asm volatile("" : "+r"(ol));
+    const int oe = (int)(xh >> 20) + 1023 - ex;  // the result's exponent field
+    if (ex == 0x7ff) {
+      oh = (mh | ml) ? 0x7ff80000u : 0u;
+      ol = 0u;
+    } else if (oe >= 2047) {
+      oh = 0x7ff00000u;
+      ol = 0u;
+    } else if (oe <= 0) {  // subnormal, by one or two bits
+      const uint32_t g = (xh & 0x000fffffu) | 0x00100000u;
+      ol = __funnelshift_r(ol, g, 1 - oe);
+      oh = g >> (1 - oe);
+    }
+  }
+  return __hiloint2double((int)(oh | sign), (int)ol);
+#else
+  return 1.0 / p;
+#endif
 }
 
 // x > 0 for a double (false for NaN), on its bits
