@@ -60,6 +60,7 @@ __global__ void __launch_bounds__(kHistThreads) radix_hist_kernel(const int32_t 
                                                                   int64_t n_cells, int shift, int bits,
                                                                   int64_t tile_stride,
                                                                   uint32_t *__restrict__ counts) {
+  grid_wait(cell_of, keys, counts);
   __shared__ uint32_t h[kHistTiles][kMaxRadix];
   const int radix = 1 << bits;
   const uint32_t mask = (uint32_t)(radix - 1);
@@ -134,6 +135,7 @@ __global__ void __launch_bounds__(32 * kScanDigits) scan_tiles_kernel(const uint
                                                                       int64_t n_tiles, int64_t tile_stride,
                                                                       int64_t part, uint32_t *__restrict__ pos,
                                                                       uint32_t *__restrict__ totals) {
+  grid_wait(counts, pos, totals);
   __shared__ uint32_t out[kScanChunk][kScanDigits + 1];  // [tile][digit]
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int d0 = blockIdx.x * kScanDigits, d = d0 + w;
@@ -209,6 +211,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) radix_scatter_kernel(
     const int32_t *__restrict__ cell_of, const uint32_t *__restrict__ keys_in, const int32_t *__restrict__ idx_in,
     int64_t n, int64_t n_cells, int shift, int bits, const uint32_t *__restrict__ pos,
     const uint32_t *__restrict__ totals, uint32_t *__restrict__ keys_out, int32_t *__restrict__ idx_out) {
+  grid_wait(cell_of, keys_in, idx_in, pos, totals, keys_out, idx_out);
   // the per-warp digit counts are dead once every key knows its place, so
   // the tile staged sorted by digit reuses their memory
   constexpr int kCountBytes = kSortWarps * kMaxRadix * 2, kStageBytes = kSortTile * 8;
@@ -339,6 +342,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) radix_scatter_kernel(
 constexpr int kOffItems = 8;
 __global__ void __launch_bounds__(256) cell_offsets_kernel(const uint32_t *__restrict__ keys, int64_t n,
                                                            int64_t n_cells, int64_t *__restrict__ offsets) {
+  grid_wait(keys, offsets);
   constexpr int kR = kOffItems / 4;
   const int lane = threadIdx.x & 31;
   const int64_t i0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (32 * kOffItems) + 4 * lane;
@@ -383,6 +387,7 @@ template <typename VT>
 __global__ void __launch_bounds__(256) gather_sorted_kernel(const VT *__restrict__ v, int64_t n,
                                                             const int32_t *__restrict__ perm, VT *__restrict__ v_sorted,
                                                             int vec) {
+  grid_wait(v, perm, v_sorted);
   const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
   if (i >= n) return;
   if (i + 4 <= n) {
@@ -418,6 +423,7 @@ __global__ void __launch_bounds__(256) gather_sorted_kernel(const VT *__restrict
 template <typename VT>
 __global__ void __launch_bounds__(256) copy_tail_kernel(const VT *__restrict__ v, VT *__restrict__ v_out, int64_t n,
                                                         const int64_t *__restrict__ first) {
+  grid_wait(v, v_out, first);
   const int64_t a = *first;
   for (int64_t i = a + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     v_out[i] = v[i];
@@ -429,9 +435,9 @@ __global__ void __launch_bounds__(256) copy_tail_kernel(const VT *__restrict__ v
 void launch_copy_tail(const void *v, void *v_out, int v_dtype, int64_t n, const int64_t *first, cudaStream_t st) {
   if (n <= 0) return;
   if (v_dtype == FP_V_F32)
-    copy_tail_kernel<float><<<304, 256, 0, st>>>((const float *)v, (float *)v_out, n, first);
+    launch_after(copy_tail_kernel<float>, 304, 256, 0, st, (const float *)v, (float *)v_out, n, first);
   else
-    copy_tail_kernel<double><<<304, 256, 0, st>>>((const double *)v, (double *)v_out, n, first);
+    launch_after(copy_tail_kernel<double>, 304, 256, 0, st, (const double *)v, (double *)v_out, n, first);
 }
 
 static inline size_t sort_align(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -492,29 +498,30 @@ void launch_sort_by_cell(const int32_t *cell_of, int64_t n, int64_t n_cells, int
     const int bits = P.bits[q], radix = 1 << bits;
     if (n > 0) {
       if (q == 0)
-        radix_hist_kernel<true><<<(unsigned)P.hist_blocks, kHistThreads, 0, st>>>(cell_of, nullptr, n, n_cells, shift,
-                                                                                  bits, P.tile_stride, counts);
+        launch_after(radix_hist_kernel<true>, (unsigned)P.hist_blocks, kHistThreads, 0, st, cell_of, nullptr, n,
+                     n_cells, shift, bits, P.tile_stride, counts);
       else
-        radix_hist_kernel<false><<<(unsigned)P.hist_blocks, kHistThreads, 0, st>>>(
-            nullptr, keys[cur], n, n_cells, shift, bits, P.tile_stride, counts);
+        launch_after(radix_hist_kernel<false>, (unsigned)P.hist_blocks, kHistThreads, 0, st, nullptr, keys[cur], n,
+                     n_cells, shift, bits, P.tile_stride, counts);
       const int64_t chunks = (P.n_tiles + kScanChunk - 1) / kScanChunk;
       const int64_t part = (chunks + kScanParts - 1) / kScanParts * kScanChunk;
       const dim3 grid((unsigned)((radix + kScanDigits - 1) / kScanDigits), (unsigned)((P.n_tiles + part - 1) / part));
-      scan_tiles_kernel<<<grid, 32 * kScanDigits, 0, st>>>(counts, radix, P.n_tiles, P.tile_stride, part, pos, totals);
+      launch_after(scan_tiles_kernel, grid, 32 * kScanDigits, 0, st, counts, radix, P.n_tiles, P.tile_stride, part,
+                   pos, totals);
       // the last pass writes the permutation straight into perm
       int32_t *idx_dst = q == P.passes - 1 ? perm : idx[cur ^ 1];
       if (q == 0)
-        radix_scatter_kernel<true><<<(unsigned)P.n_tiles, kSortThreads, 0, st>>>(
-            cell_of, nullptr, nullptr, n, n_cells, shift, bits, pos, totals, keys[cur ^ 1], idx_dst);
+        launch_after(radix_scatter_kernel<true>, (unsigned)P.n_tiles, kSortThreads, 0, st, cell_of, nullptr, nullptr,
+                     n, n_cells, shift, bits, pos, totals, keys[cur ^ 1], idx_dst);
       else
-        radix_scatter_kernel<false><<<(unsigned)P.n_tiles, kSortThreads, 0, st>>>(
-            nullptr, keys[cur], idx[cur], n, n_cells, shift, bits, pos, totals, keys[cur ^ 1], idx_dst);
+        launch_after(radix_scatter_kernel<false>, (unsigned)P.n_tiles, kSortThreads, 0, st, nullptr, keys[cur],
+                     idx[cur], n, n_cells, shift, bits, pos, totals, keys[cur ^ 1], idx_dst);
     }
     cur ^= 1;
     shift += bits;
   }
   const int64_t blocks = (n + 1 + 256 * kOffItems - 1) / (256 * kOffItems);
-  cell_offsets_kernel<<<(unsigned)blocks, 256, 0, st>>>(keys[cur], n, n_cells, offsets);
+  launch_after(cell_offsets_kernel, (unsigned)blocks, 256, 0, st, keys[cur], n, n_cells, offsets);
   if (sorted_keys) *sorted_keys = keys[cur];
 }
 
@@ -525,10 +532,11 @@ void launch_gather_sorted(const void *v, int v_dtype, int64_t n, const int32_t *
   const int vec = quad_classes(v_sorted, v_sorted, n, 0, v_dtype == FP_V_F32 ? 4 : 8) |
                   (((uintptr_t)perm & 15) == 0 ? 64 : 0);
   if (v_dtype == FP_V_F32)
-    gather_sorted_kernel<float><<<(unsigned)blocks, 256, 0, st>>>((const float *)v, n, perm, (float *)v_sorted, vec);
+    launch_after(gather_sorted_kernel<float>, (unsigned)blocks, 256, 0, st, (const float *)v, n, perm,
+                 (float *)v_sorted, vec);
   else
-    gather_sorted_kernel<double><<<(unsigned)blocks, 256, 0, st>>>((const double *)v, n, perm, (double *)v_sorted,
-                                                                   vec);
+    launch_after(gather_sorted_kernel<double>, (unsigned)blocks, 256, 0, st, (const double *)v, n, perm,
+                 (double *)v_sorted, vec);
 }
 
 }  // namespace fpc
