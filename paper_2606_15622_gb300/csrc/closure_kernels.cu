@@ -359,7 +359,7 @@ void launch_solve(const double *mom, const double *tau, int64_t n_cells, const f
   const unsigned three = (unsigned)(blocks < 3 * sm_count() ? blocks : 3 * sm_count());
   // a half warp a cell while every SM sub-partition has one warp of them at
   // most (eight times the FP64 instructions a cell, half the chain): 400 cells
-  // 13.4 us (a thread a cell 25.3 when this took 16.5)
+  // 12.5 us (a thread a cell 25.3 when this took 16.5)
   const bool few = n_cells <= 8 * (int64_t)sm_count();
   if (lu)
     solve_kernel<true><<<two, threads, 0, st>>>(mom, tau, n_cells, prm, coeffs, flags, lu);

@@ -233,7 +233,7 @@ __device__ __forceinline__ int pivoted_solve(double (&a)[9][10], double rtol, do
   for (int k = 8; k >= 0; --k) {
     double s = a[k][9];
 #pragma unroll
-    for (int j = k + 1; j < 9; ++j) s = fma(-a[k][j], y[j], s);
+    for (int j = 8; j > k; --j) s = fma(-a[k][j], y[j], s);  // as they become known (closure_cell_group16)
     y[k] = s * rinv[k];
   }
   return flag;
@@ -651,7 +651,7 @@ __device__ __forceinline__ int closure_cell_mixed(const double *__restrict__ mc,
 // shuffles, and each lane eliminates its own row; the back substitution
 // broadcasts each y_k from lane k.  Every entry sees the operations of
 // closure_cell in the same order (the same emitted expressions, multipliers
-// a_iK * (1 / a_KK), fma updates, the sum over j ascending), so coefficients
+// a_iK * (1 / a_KK), fma updates, the sum over j descending), so coefficients
 // and flags are identical; what changes is the length of the dependent chain
 // (FP64 instructions have a latency of about 64 cycles on this GPU, a
 // reciprocal by rcp_d about 400), roughly halved, which is what a short
@@ -725,12 +725,11 @@ __device__ __forceinline__ int closure_cell_group16(const double *__restrict__ m
       for (int j = K + 1; j < 10; ++j) row[j] = fma(-l, piv[j], row[j]);
     }
   }
+  double s = row[9];
 #pragma unroll
   for (int k = 8; k >= 0; --k) {
-    double s = row[9];
-#pragma unroll
-    for (int j = k + 1; j < 9; ++j) s = fma(-row[j], y[j], s);
     y[k] = __shfl_sync(kAll, s * rinv[k], k, 16);
+    s = fma(-row[k], y[k], s);  // every row's sum at once; the rows above k go on to use it
   }
   if (!fl) {
     fl = sfl;
