@@ -22,6 +22,7 @@ class ClosureFunction(torch.autograd.Function):
         ctx.save_for_backward(v, offsets, tau, mom, y, fl)
         ctx.params = params
         ctx.mark_non_differentiable(fl)
+        ctx.set_materialize_grads(False)  # an output without a gradient gives None, not a tensor of zeros
         return mom, y, fl
 
     @staticmethod
