@@ -260,31 +260,58 @@ static __device__ __noinline__ void solve_own(int64_t c, const double *__restric
   flags[c] = fl;
 }
 
+// The moment rows of nc <= 32 consecutive cells into shared memory, row l at l
+// kRowStride (odd: the lanes read their own rows without bank conflicts), by
+// contiguous loads of the calling warp: a lane that read its own row from
+// global memory would touch a line a load.
+constexpr int kRowStride = FP_NMOM | 1;
+__device__ __forceinline__ void load_rows(const double *__restrict__ src, int nc, double *row, int lane) {
+  double x[FP_NMOM];
+#pragma unroll
+  for (int k = 0; k < FP_NMOM; ++k) x[k] = 32 * k + lane < nc * FP_NMOM ? src[32 * k + lane] : 0.0;
+#pragma unroll
+  for (int k = 0; k < FP_NMOM; ++k) {
+    const int i = 32 * k + lane;
+    row[i + i / FP_NMOM * (kRowStride - FP_NMOM)] = x[k];
+  }
+}
+
 // The mixed-precision solve, one thread per cell; cells that it refuses are
-// solved by their warp.  Three blocks per SM: bound by the dependent chains
-// of the FP32 elimination and the selects of its row swaps.
-// 131,072 cells of 91 particles: 70 us (97 with the residual in FP64 and a
-// single-lane fallback), 16,384 of 50: 29 (36.5);
-// two or four blocks per SM 75 / 72.
-__global__ void __launch_bounds__(128, 3) solve_mixed_kernel(const double *__restrict__ mom,
+// solved by their warp.  Bound by the dependent chains of the FP32 elimination
+// and the selects of its row swaps, so four blocks per SM (spilling some of
+// the system), and the rows staged: read twice by each lane from global memory
+// they took some 26 us of the load pipe.
+// 131,072 cells of 91 particles: 53 us; 65 with three blocks, 69 two, 56 five,
+// 72 without the staging (three or four), 97 with the residual in FP64 and a
+// single-lane fallback.  16,384 cells of 50: 23.4 (27.5 without, 36.5).  (The
+// FP64 solves gain nothing by it: 107 us against 100.)
+__global__ void __launch_bounds__(128, 4) solve_mixed_kernel(const double *__restrict__ mom,
                                                              const double *__restrict__ tau, int64_t n_cells,
                                                              SolveParams prm, double *__restrict__ coeffs,
                                                              int32_t *__restrict__ flags) {
+  __shared__ double rows[4][32 * kRowStride];
   const int lane = threadIdx.x & 31;
+  double *row = rows[threadIdx.x >> 5];
   for (int64_t c0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; c0 < n_cells;
        c0 += (int64_t)gridDim.x * blockDim.x) {
     const int64_t c = c0 + lane;
+    const int nc = (int)(n_cells - c0 < 32 ? n_cells - c0 : 32);
+    load_rows(mom + c0 * FP_NMOM, nc, row, lane);
+    __syncwarp();
     bool todo = false;
+    double y[9] = {};
     if (c < n_cells) {
-      double y[9];
-      const int fl = closure_cell_mixed(mom + c * FP_NMOM, tau[c], prm, y, todo);
-      if (!todo) {
-        double *yc = coeffs + c * 9;
-#pragma unroll
-        for (int q = 0; q < 9; ++q) yc[q] = y[q];
-        flags[c] = fl;
-      }
+      const int fl = closure_cell_mixed(row + lane * kRowStride, tau[c], prm, y, todo);
+      if (!todo) flags[c] = fl;
     }
+    // the coefficients leave by contiguous stores (zeros for the cells that the
+    // FP64 solve below overwrites)
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 9; ++q) row[lane * 9 + q] = todo ? 0.0 : y[q];
+    __syncwarp();
+    for (int i = lane; i < nc * 9; i += 32) coeffs[c0 * 9 + i] = row[i];
+    __syncwarp();
     const unsigned list = __ballot_sync(0xffffffffu, todo);
     if (__popc(list) > 4) {
       if (todo) solve_own(c, mom, tau, prm, coeffs, flags);
@@ -356,7 +383,7 @@ void launch_solve(const double *mom, const double *tau, int64_t n_cells, const f
   const int threads = 128;
   const int64_t blocks = (n_cells + threads - 1) / threads;
   const unsigned two = (unsigned)(blocks < 2 * sm_count() ? blocks : 2 * sm_count());
-  const unsigned three = (unsigned)(blocks < 3 * sm_count() ? blocks : 3 * sm_count());
+  const unsigned four = (unsigned)(blocks < 4 * sm_count() ? blocks : 4 * sm_count());
   // a half warp a cell while every SM sub-partition has one warp of them at
   // most (eight times the FP64 instructions a cell, half the chain): 400 cells
   // 12.5 us (a thread a cell 25.3 when this took 16.5)
@@ -364,7 +391,7 @@ void launch_solve(const double *mom, const double *tau, int64_t n_cells, const f
   if (lu)
     solve_kernel<true><<<two, threads, 0, st>>>(mom, tau, n_cells, prm, coeffs, flags, lu);
   else if (prec == FP_PREC_FP32_MOMENTS)  // FP32-accurate moments: the mixed-precision solve
-    solve_mixed_kernel<<<three, threads, 0, st>>>(mom, tau, n_cells, prm, coeffs, flags);
+    solve_mixed_kernel<<<four, threads, 0, st>>>(mom, tau, n_cells, prm, coeffs, flags);
   else if (few)
     solve_group_kernel<<<(unsigned)((n_cells + 7) / 8), threads, 0, st>>>(mom, tau, n_cells, prm, coeffs, flags);
   else

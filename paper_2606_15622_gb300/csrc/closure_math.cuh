@@ -349,6 +349,18 @@ struct F2 {
   float h, l;
 };
 
+// double -> FP32 rounded to nearest even, by integers and selects; values of
+// 2^127 and more infinite (a system that holds one is refused), below 2^-126
+// zero.  (d2f_rn branches: 56.0 against 53.5 us for 131,072 cells.)
+__device__ __forceinline__ float narrow_select(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t a = hi & 0x7fffffffu;
+  uint32_t u = __funnelshift_l(lo, hi, 3) - (896u << 23);
+  u += ((lo & 0x1fffffffu) + 0x0fffffffu + (u & 1u)) >> 29;
+  u = a < (897u << 20) ? 0u : a >= (1150u << 20) ? 0x7f800000u : u & 0x7fffffffu;
+  return __uint_as_float(u | (hi & 0x80000000u));
+}
+
 // double -> F2 on the integer pipe: the leading 24 bits truncated, the other 29
 // rounded to FP32.  For |x| < 2^100; below 2^-74 without the low bits, below
 // 2^-120 zero.
@@ -584,7 +596,7 @@ __device__ __forceinline__ int closure_cell_mixed(const double *__restrict__ mc,
     for (int k = 0; k < FP_NMOM; ++k) fin = fin && finite_d(mc[k]);
     if (!fin) fl |= FP_FLAG_NONFINITE;
     if (mc[kN] < (double)prm.min_particles) fl |= FP_FLAG_FEW;
-    if (!(mc[kTheta] > 0.0)) fl |= FP_FLAG_SINGULAR;
+    if (!positive_d(mc[kTheta])) fl |= FP_FLAG_SINGULAR;
     if (!fl && mc[kN] < (double)prm.min_regular) fl |= FP_FLAG_SINGULAR;
     auto near_one = [](double v) { return (((uint32_t)__double2hiint(v) >> 20) & 0x7ffu) - (1023u - 20u) < 40u; };
     in_range = near_one(tc) && near_one(mc[kTheta]);
@@ -598,7 +610,7 @@ __device__ __forceinline__ int closure_cell_mixed(const double *__restrict__ mc,
   {
     float mf[FP_NMOM];
 #pragma unroll
-    for (int k = 0; k < FP_NMOM; ++k) mf[k] = d2f_rn(mc[k]);
+    for (int k = 0; k < FP_NMOM; ++k) mf[k] = narrow_select(mc[k]);
 #pragma unroll
     for (int r = 0; r < 9; ++r)
 #pragma unroll
