@@ -43,12 +43,10 @@ if ROOT not in sys.path:
 
 METRIC = "closure cells/s + particles/s (exact FP64, FP32-moment, surrogate) at stated C/Gamma error"
 L2_FLUSH_BYTES = 256 << 20
-# DRAM bytes (read + write) per launch on this workload, from one ncu capture
-# of the current build of each kernel; None once a kernel has changed since
 # DRAM bytes (read + write) of one launch in the ncu captures summarised under
 # profiles/ (current kernels; a kernel changed since its capture has none)
-NCU_DRAM_BYTES = {"velocity_update": 298.03e6, "gather_fp32": 175.77e6, "solve_fp64": 85.43e6,
-                  "gather_fp64": 313.65e6}
+NCU_DRAM_BYTES = {"velocity_update": 298.03e6, "gather_fp32": 175.77e6, "solve_mixed": 34.37e6,
+                  "gather_fp64": 326.46e6}
 ORACLE_BLOCK = 4096            # cells per block of the CPU oracle's timing
 E2E_CHUNKS = 8                 # chunks of the host-resident step (copy / compute overlap)
 WEIGHTS = os.path.join(ROOT, "paper_2606_15622_gb300", "weights", "surrogate_full.fpw")
@@ -61,10 +59,10 @@ LITE_BYTES_PER_CELL = 8 + 8 * 14        # one offset read, the LITE moment vecto
 VEL_BYTES_PER_PARTICLE = 24             # read + write three FP32 components
 VEL_BYTES_PER_CELL = 8 + 8 * (3 + 1 + 3 + 9 + 1) + 4 + 4 + 8  # offset; U, theta, q, C, Gamma, tau; flags in/out; alpha
 GATHER64_FLOPS_PER_PARTICLE = 61       # FP64 gather: 3 (mean) + 3 (centre) + 55 (26 monomial sums, FMA = 2)
-SOLVE_MIXED_FP64_FLOPS_PER_CELL = 290  # mixed solve, FP64 part: the emitted entries (~150), b - A x (~135, FMA = 2), update
 SOLVE_FLOPS_PER_CELL = 658              # FP64: assembly + elimination + back substitution (FMA = 2)
 MLP_FLOPS_PER_CELL = 2 * (32 * 128 + 3 * 128 * 128 + 128 * 16)  # padded layer shapes
 FP64_PEAK_TFLOPS = 1.197                # FP64 peak of a GB300, measured with independent DFMA chains
+FP32_PEAK_TFLOPS = 73.7                 # FP32 peak, measured with independent FFMA chains
 
 
 def _peaks():
@@ -390,16 +388,16 @@ def run_ours(args):
                                               "peak_note": "FP64 pipe, measured FMA chain"}),
         "velocity_update": kern(t_vel, "hbm", vel_bytes / (t_vel * 1e-3) / 1e9, "GB/s", peaks["hbm_gbs"],
                                 {"algorithmic_bytes": vel_bytes}),
-        "solve_mixed": kern(t_solve_mixed, "alu", SOLVE_MIXED_FP64_FLOPS_PER_CELL * n_cells / (t_solve_mixed * 1e-3) / 1e12,
-                            "TFLOP/s", FP64_PEAK_TFLOPS,
-                            {"algorithmic_flops": SOLVE_MIXED_FP64_FLOPS_PER_CELL * n_cells,
-                             "peak_note": "FP64 part only (FP64 assembly of the residual, refinement); the FP32 "
-                                          "factorisation and solves run on the FP32 pipe"}),
+        "solve_mixed": kern(t_solve_mixed, "alu", SOLVE_FLOPS_PER_CELL * n_cells / (t_solve_mixed * 1e-3) / 1e12,
+                            "TFLOP/s", FP32_PEAK_TFLOPS,
+                            {"algorithmic_flops": SOLVE_FLOPS_PER_CELL * n_cells,
+                             "peak_note": "FP32 pipe, measured FMA chain; one elimination's flops (the residual in "
+                                          "pairs of FP32 and the correction are not counted)"}),
         "gather_fp64": kern(t_g64, "alu", GATHER64_FLOPS_PER_PARTICLE * n_p / (t_g64 * 1e-3) / 1e12, "TFLOP/s",
                             FP64_PEAK_TFLOPS, {"algorithmic_flops": GATHER64_FLOPS_PER_PARTICLE * n_p,
-                                               "peak_note": "FP64 pipe, measured FMA chain; an FP64 add or multiply "
-                                                            "takes the pipe slot of an FMA, and idle lanes of a warp "
-                                                            "instruction take it too (ncu: FP64 pipe 89 % busy)"}),
+                                               "peak_note": "FP64 pipe, measured FMA chain; the central sums run in "
+                                                            "58-bit fixed point on the integer pipes instead, so the "
+                                                            "fraction may exceed one"}),
         "mlp_forward": kern(t_mlp, "tensor", MLP_FLOPS_PER_CELL * n_cells / (t_mlp * 1e-3) / 1e12, "TFLOP/s",
                             peaks["bf16_tflops"], {"algorithmic_flops": MLP_FLOPS_PER_CELL * n_cells}),
     }
@@ -640,7 +638,7 @@ def run_ours(args):
             "exact_fp32_moments": {"ms": round(t_exact32, 5),
                                    "cells_per_s": round(n_cells / (t_exact32 * 1e-3), 1),
                                    "particles_per_s": round(n_p / (t_exact32 * 1e-3), 1),
-                                   "solve": "mixed precision (FP32 factors, FP64 residual, one refinement; "
+                                   "solve": "mixed precision (FP32 factors, residual in FP32 pairs, one refinement; "
                                             "agrees with the FP64 solve to <= 4e-9 on the cylinder)",
                                    "with_factors_for_the_adjoint_ms": round(per_call["exact_closure"], 5),
                                    "error_vs_oracle": "<= 1e-4 relative, or kappa * 2^-24 on 7 of 131,021 "
