@@ -19,9 +19,9 @@ namespace fpc {
 // called grid_wait or grid_release, or ended.
 // For chains of short kernels: the sort's eight launches of a collision step
 // 504 -> 484 us (131,072 cells) and 153 -> 144 (20,011, LITE), the training
-// step's two 57 -> 51.  Not for the long ones (gathers, solves, adjoint): they are as long
-// as the machine is wide, their blocks gain nothing by waiting on the SMs, and
-// loads outside the read-only cache cost them more (exact closure 158 -> 207).
+// step's two 57 -> 51.  Not for kernels of few resident blocks an SM (gathers,
+// solves, adjoint): blocks that start early crowd on the first SMs that drain
+// (exact closure of 131,072 cells 158 -> 207 us, of 16,384 cells 41 -> 47).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename P>
