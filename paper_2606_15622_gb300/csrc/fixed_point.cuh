@@ -32,6 +32,10 @@ constexpr int kFxBits = 58;   // fraction bits: |c| < 2^58 units
 constexpr int kFxLimb = 29;   // bits of the low limb
 constexpr int kFxMid = 15;    // particles a lane sums before its middle sums (terms h l' + l h' < 2^59) are carried
 constexpr int kFxBlock = 30;  // .. and before all its sums (terms < 2^58) are folded
+constexpr int kFxFold = 3;    // bits a folded sum drops, so that ..
+constexpr int kFxLanes = 8;   // .. the folded sums of so many lanes add up in 64 bits (more lanes: in FP64 from there)
+static_assert(kFxBlock < 1 << (63 - kFxBits), "a lane's block of terms below 2^kFxBits");
+static_assert(kFxLanes * kFxBlock < 1 << (63 - kFxBits + kFxFold), "the folded blocks of kFxLanes lanes");
 // binades the largest |v| may lie above E (the mantissa, shifted to bit 63,
 // is only ever shifted right)
 constexpr int kFxHead = 63 - kFxBits;
@@ -182,9 +186,9 @@ struct FxSums {
   // a term, goes into the middle sums beforehand (<|c|^6> sums its own), and
   // so do the halves that make the shifts of fx_fold round
   FPC_HD void clear(int count) {
-    for (int q = 0; q < 6; ++q) P[q] = 4;
+    for (int q = 0; q < 6; ++q) P[q] = 1 << (kFxFold - 1);
     for (int q = 0; q < kN; ++q) {
-      H[q] = 4;
+      H[q] = 1 << (kFxFold - 1);
       M[q] = ((int64_t)(q == 19 ? 0 : count) << (kFxLimb - 2)) + ((int64_t)1 << (kFxLimb - 1));
     }
     L = 0;
@@ -227,16 +231,16 @@ FPC_HD void fx_accumulate(FxSums<kM6> &S, int64_t cx, int64_t cy, int64_t cz, co
   }
 }
 
-// The lane's sum of slot q (0..25, the order of the gathered sums), an eighth
-// of its unit (room for the lanes of a cell): the sum is 2^s times it with
-// s = 3 - kFxBits + a e0 + b e1 + c e2 + d er
+// The lane's sum of slot q (0..25, the order of the gathered sums) without its
+// kFxFold lowest bits (room for kFxLanes lanes, no more): the sum is 2^s times
+// it with s = kFxFold - kFxBits + a e0 + b e1 + c e2 + d er
 template <bool kM6>
 FPC_HD int64_t fx_fold(const FxSums<kM6> &S, int q) {
-  if (q < 6) return S.P[q] >> 3;
+  if (q < 6) return S.P[q] >> kFxFold;
   const int j = q - 6;
   if (j >= FxSums<kM6>::kN) return 0;
   const int64_t m = j == 19 ? S.M[j] + (S.L >> kFxLimb) : S.M[j];
-  return (S.H[j] + (m >> kFxLimb)) >> 3;
+  return (S.H[j] + (m >> kFxLimb)) >> kFxFold;
 }
 
 // a | b << 8 | c << 16 | d << 24 of slot q
@@ -255,7 +259,7 @@ FPC_HD uint32_t fx_weights(int q) {
   return 3 * R;
 }
 FPC_HD int fx_exponent(uint32_t w, const FxCell &c) {
-  return 3 - kFxBits + (int)(w & 255u) * c.e[0] + (int)((w >> 8) & 255u) * c.e[1] + (int)((w >> 16) & 255u) * c.e[2] +
+  return kFxFold - kFxBits + (int)(w & 255u) * c.e[0] + (int)((w >> 8) & 255u) * c.e[1] + (int)((w >> 16) & 255u) * c.e[2] +
          (int)(w >> 24) * c.er;
 }
 

@@ -94,16 +94,19 @@ constexpr int kOwn = 4;
 __device__ __forceinline__ int own_slot(int k, int lg) { return 16 * (k >> 1) + 2 * (lg & 7) + (k & 1); }
 
 // The 26 slots of the group's G lanes summed, each by the lanes that own it
-// (G = 32: four lanes).  get(q) is the lane's own slot q (q a constant after
-// unrolling).  sc: the warp's scratch (32 rows of 128 bytes, the chunks of a
-// row rotated so that a quarter-warp's 16-byte accesses hit all banks).
+// (G = 32: four lanes): eight lanes' in T, the eights in FP64 (integer sums
+// have room for kFxLanes lanes).  get(q) is the lane's own slot q (q a
+// constant after unrolling).  sc: the warp's scratch (32 rows of 128 bytes, the
+// chunks of a row rotated so that a quarter-warp's 16-byte accesses hit all
+// banks).
 template <int G, typename T, class Get>
-__device__ __forceinline__ void group_transpose(Get get, T (&out)[kOwn], T *sc, int lane) {
+__device__ __forceinline__ void group_transpose(Get get, double (&out)[kOwn], T *sc, int lane) {
   static_assert(sizeof(T) == 8, "two slots a 16-byte chunk");
   struct alignas(16) Two {
     T a, b;
   };
   constexpr int kRows = 8;  // rows a lane adds
+  static_assert(kRows == kFxLanes, "integer sums of so many lanes");
   Two *s2 = reinterpret_cast<Two *>(sc);
   const int ch = lane & 7, base = lane & ~7;
 #pragma unroll
@@ -114,7 +117,7 @@ __device__ __forceinline__ void group_transpose(Get get, T (&out)[kOwn], T *sc, 
       if (q < kNSum) s2[lane * 8 + (w ^ ch)] = Two{get(q), get(q + 1)};
     }
     __syncwarp();
-    T a = 0, b = 0;
+    double a = 0.0, b = 0.0;
     if (16 * half + 2 * ch < kNSum) {
       T ra[kRows], rb[kRows];
 #pragma unroll
@@ -130,8 +133,8 @@ __device__ __forceinline__ void group_transpose(Get get, T (&out)[kOwn], T *sc, 
           ra[i] += ra[i + o];
           rb[i] += rb[i + o];
         }
-      a = ra[0];
-      b = rb[0];
+      a = (double)ra[0];
+      b = (double)rb[0];
     }
 #pragma unroll
     for (int o = 8; o < G; o <<= 1) {
@@ -263,13 +266,10 @@ __global__ void __launch_bounds__(32 * kGWarps, kGBlocksPerSm)
             fx_accumulate<kM6>(S, in ? fx_from_words(wx.x, wx.y, t0) - U0 : 0, in ? fx_from_words(wy.x, wy.y, t1) - U1 : 0,
                                in ? fx_from_words(wz.x, wz.y, t2) - U2 : 0, cell);
           }
-          int64_t f[kOwn];
+          double f[kOwn];
           group_transpose<G, int64_t>([&](int q) { return fx_fold<kM6>(S, q); }, f, sc, lane);
 #pragma unroll
-          for (int k = 0; k < kOwn; ++k) {
-            const double d = (double)f[k];
-            val[k] = b0 == 0 ? d : val[k] + d;
-          }
+          for (int k = 0; k < kOwn; ++k) val[k] = b0 == 0 ? f[k] : val[k] + f[k];
         }
       }
       if (!__all_sync(0xffffffffu, fx || n == 0)) {  // some cell of the task in FP64
