@@ -78,7 +78,7 @@ FPC_HD int64_t fx_sqr(Fx a) {
 // Finite v = (-1)^s 1.f 2^e (the double's two words) in units of
 // 2^(E - 58), modulo 2^64, truncated; top = E + kFxHead + 1023, e <= E + kFxHead.
 // Zeros and subnormals (whose shift leaves nothing for an accepted E) give 0.
-FPC_HD int64_t fx_from_words(uint32_t hi, uint32_t lo, int top) {
+FPC_HD uint64_t fx_from_words(uint32_t hi, uint32_t lo, int top) {
   // the mantissa 1.f to bits 63 .. 11, then down by the binades to 2^(E + kFxHead)
   const uint64_t m = ((uint64_t)(hi | 0x00100000u) << 43) | ((uint64_t)lo << 11);
   const int r = top - (int)((hi >> 20) & 0x7ffu);
@@ -88,9 +88,11 @@ FPC_HD int64_t fx_from_words(uint32_t hi, uint32_t lo, int top) {
 #else
   const uint64_t u = r > 63 ? 0 : m >> r;
 #endif
-  const int64_t s = -(int64_t)(hi >> 31);
-  return (int64_t)(u ^ (uint64_t)s) - s;
+  const uint64_t s = 0ull - (uint64_t)(hi >> 31);
+  return (u ^ s) - s;
 }
+// c = v - U of such positions: they wrap, their difference is below 2^kFxBits
+FPC_HD int64_t fx_offset(uint64_t v, uint64_t U) { return (int64_t)(v - U); }
 
 // order of doubles on their high words: a signed key
 FPC_HD int32_t fx_key(uint32_t hi) { return (int32_t)(hi ^ (uint32_t)(((int32_t)hi >> 31) & 0x7fffffff)); }

@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(32 * kGWarps, kGBlocksPerSm)
       uint32_t mh;
       const bool fixed = (fx_range(U, klo, khi, mh) && n > kGFew) || (lg & 3) == 3;
       const uint2 uw = v_words(U);
-      const int64_t Uf = fx_from_words(uw.x, uw.y, fx_exp(mh) + kFxHead + 1023);
+      const uint64_t Uf = fx_from_words(uw.x, uw.y, fx_exp(mh) + kFxHead + 1023);
       const unsigned okmask = __ballot_sync(0xffffffffu, fixed);
       const bool fx = ((~okmask >> gbase) & (0xffffffffu >> (32 - G))) == 0u;  // the whole cell
       const FxCell cell = fx_cell(__shfl_sync(0xffffffffu, mh, gbase), __shfl_sync(0xffffffffu, mh, gbase + 1),
@@ -241,8 +241,9 @@ __global__ void __launch_bounds__(32 * kGWarps, kGBlocksPerSm)
       double val[kOwn] = {};  // the sums of this lane's slots
       // ---- pass B ----
       {
-        const int64_t U0 = __shfl_sync(0xffffffffu, Uf, gbase), U1 = __shfl_sync(0xffffffffu, Uf, gbase + 1),
-                      U2 = __shfl_sync(0xffffffffu, Uf, gbase + 2);
+        const uint64_t U0 = __shfl_sync(0xffffffffu, (unsigned long long)Uf, gbase),
+                       U1 = __shfl_sync(0xffffffffu, (unsigned long long)Uf, gbase + 1),
+                       U2 = __shfl_sync(0xffffffffu, (unsigned long long)Uf, gbase + 2);
         const int t0 = cell.e[0] + kFxHead + 1023, t1 = cell.e[1] + kFxHead + 1023, t2 = cell.e[2] + kFxHead + 1023;
         const int nf = fx ? n : 0;
         const int itfx = __reduce_max_sync(0xffffffffu, (nf + G - 1) / G);
@@ -263,8 +264,9 @@ __global__ void __launch_bounds__(32 * kGWarps, kGBlocksPerSm)
             if (left > G) x = __ldg(qx), y = __ldg(qy), z = __ldg(qz);
             const bool in = left > 0;  // a lane past its cell adds c = 0
             left -= G;
-            fx_accumulate<kM6>(S, in ? fx_from_words(wx.x, wx.y, t0) - U0 : 0, in ? fx_from_words(wy.x, wy.y, t1) - U1 : 0,
-                               in ? fx_from_words(wz.x, wz.y, t2) - U2 : 0, cell);
+            fx_accumulate<kM6>(S, in ? fx_offset(fx_from_words(wx.x, wx.y, t0), U0) : 0,
+                               in ? fx_offset(fx_from_words(wy.x, wy.y, t1), U1) : 0,
+                               in ? fx_offset(fx_from_words(wz.x, wz.y, t2), U2) : 0, cell);
           }
           double f[kOwn];
           group_transpose<G, int64_t>([&](int q) { return fx_fold<kM6>(S, q); }, f, sc, lane);
@@ -292,7 +294,7 @@ __global__ void __launch_bounds__(32 * kGWarps, kGBlocksPerSm)
       for (int k = 0; k < kOwn; ++k) {
         // inv_n 2^s: a normal double times a power of two, exact
         const int s = fx ? fx_exponent(wq[k], cell) : 0;
-        out[k] = val[k] * __hiloint2double(__double2hiint(inv_n) + (n > 0 ? s << 20 : 0), __double2loint(inv_n));
+        out[k] = val[k] * __hiloint2double(__double2hiint(inv_n) + (n > 0 ? s * (1 << 20) : 0), __double2loint(inv_n));
       }
       const double u11 = __shfl_sync(0xffffffffu, out[0], gbase), u22 = __shfl_sync(0xffffffffu, out[1], gbase + 1),
                    u33 = __shfl_sync(0xffffffffu, out[1], gbase + 2);
