@@ -32,7 +32,7 @@ constexpr int kFxBits = 58;   // fraction bits: |c| < 2^58 units
 constexpr int kFxLimb = 29;   // bits of the low limb
 constexpr int kFxMid = 15;    // particles a lane sums before its middle sums (terms h l' + l h' < 2^59) are carried
 constexpr int kFxBlock = 30;  // .. and before all its sums (terms < 2^58) are folded
-constexpr int kFxFold = 3;    // bits a folded sum drops, so that ..
+constexpr int kFxFold = 3;    // bits a folded sum drops at most, so that ..
 constexpr int kFxLanes = 8;   // .. the folded sums of so many lanes add up in 64 bits (more lanes: in FP64 from there)
 static_assert(kFxBlock < 1 << (63 - kFxBits), "a lane's block of terms below 2^kFxBits");
 static_assert(kFxLanes * kFxBlock < 1 << (63 - kFxBits + kFxFold), "the folded blocks of kFxLanes lanes");
@@ -44,6 +44,14 @@ constexpr int kFxMaxExp = 120;  // |E| accepted: 2^(5 E) and 2^(6 E) stay normal
 struct Fx {
   int32_t h, l;
 };
+
+// The bits to drop for a cell whose lanes sum up to m particles a block:
+// kFxLanes m < 2^(63 - kFxBits + bits).  Dropping three always left the sums of
+// cells of 30 particles by 32 lanes up to six times as far off as FP64 sums.
+FPC_HD int fx_fold_bits(int m) {
+  static_assert(kFxLanes == 8 && kFxFold == 3 && kFxBits == 58, "the steps below");
+  return m < 4 ? 0 : m < 8 ? 1 : m < 16 ? 2 : kFxFold;
+}
 
 // a b + c, one instruction (written out: from the C++ the compiler makes
 // 64 x 64-bit products of limbs that it has just widened)
@@ -187,10 +195,10 @@ struct FxSums {
   // for count particles to come: the mean of the dropped l l', 2^(2 kFxLimb - 2)
   // a term, goes into the middle sums beforehand (<|c|^6> sums its own), and
   // so do the halves that make the shifts of fx_fold round
-  FPC_HD void clear(int count) {
-    for (int q = 0; q < 6; ++q) P[q] = 1 << (kFxFold - 1);
+  FPC_HD void clear(int count, int fold = kFxFold) {
+    for (int q = 0; q < 6; ++q) P[q] = (1 << fold) >> 1;
     for (int q = 0; q < kN; ++q) {
-      H[q] = 1 << (kFxFold - 1);
+      H[q] = (1 << fold) >> 1;
       M[q] = ((int64_t)(q == 19 ? 0 : count) << (kFxLimb - 2)) + ((int64_t)1 << (kFxLimb - 1));
     }
     L = 0;
@@ -234,15 +242,15 @@ FPC_HD void fx_accumulate(FxSums<kM6> &S, int64_t cx, int64_t cy, int64_t cz, co
 }
 
 // The lane's sum of slot q (0..25, the order of the gathered sums) without its
-// kFxFold lowest bits (room for kFxLanes lanes, no more): the sum is 2^s times
-// it with s = kFxFold - kFxBits + a e0 + b e1 + c e2 + d er
+// `fold` lowest bits (room for kFxLanes lanes, no more): the sum is 2^s times
+// it with s = fold - kFxBits + a e0 + b e1 + c e2 + d er
 template <bool kM6>
-FPC_HD int64_t fx_fold(const FxSums<kM6> &S, int q) {
-  if (q < 6) return S.P[q] >> kFxFold;
+FPC_HD int64_t fx_fold(const FxSums<kM6> &S, int q, int fold = kFxFold) {
+  if (q < 6) return S.P[q] >> fold;
   const int j = q - 6;
   if (j >= FxSums<kM6>::kN) return 0;
   const int64_t m = j == 19 ? S.M[j] + (S.L >> kFxLimb) : S.M[j];
-  return (S.H[j] + (m >> kFxLimb)) >> kFxFold;
+  return (S.H[j] + (m >> kFxLimb)) >> fold;
 }
 
 // a | b << 8 | c << 16 | d << 24 of slot q
@@ -260,8 +268,8 @@ FPC_HD uint32_t fx_weights(int q) {
   if (q < 25) return 2 * R + (q == 22 ? X : q == 23 ? Y : Z);
   return 3 * R;
 }
-FPC_HD int fx_exponent(uint32_t w, const FxCell &c) {
-  return kFxFold - kFxBits + (int)(w & 255u) * c.e[0] + (int)((w >> 8) & 255u) * c.e[1] + (int)((w >> 16) & 255u) * c.e[2] +
+FPC_HD int fx_exponent(uint32_t w, const FxCell &c, int fold = kFxFold) {
+  return fold - kFxBits + (int)(w & 255u) * c.e[0] + (int)((w >> 8) & 255u) * c.e[1] + (int)((w >> 16) & 255u) * c.e[2] +
          (int)(w >> 24) * c.er;
 }
 

@@ -235,6 +235,7 @@ __global__ void __launch_bounds__(32 * kGWarps, kGBlocksPerSm)
       const uint64_t Uf = fx_from_words(uw.x, uw.y, fx_exp(mh) + kFxHead + 1023);
       const unsigned okmask = __ballot_sync(0xffffffffu, fixed);
       const bool fx = ((~okmask >> gbase) & (0xffffffffu >> (32 - G))) == 0u;  // the whole cell
+      const int fold = fx_fold_bits((n + G - 1) / G);
       const FxCell cell = fx_cell(__shfl_sync(0xffffffffu, mh, gbase), __shfl_sync(0xffffffffu, mh, gbase + 1),
                                   __shfl_sync(0xffffffffu, mh, gbase + 2));
 
@@ -253,7 +254,7 @@ __global__ void __launch_bounds__(32 * kGWarps, kGBlocksPerSm)
           // (loads one particle ahead)
           const VT *qx = px + b0 * G + lg, *qy = py + b0 * G + lg, *qz = pz + b0 * G + lg;
           int left = nf - b0 * G - lg;
-          S.clear(max(0, min(kFxBlock, (left + G - 1) / G)));
+          S.clear(max(0, min(kFxBlock, (left + G - 1) / G)), fold);
           VT x = VT(0), y = VT(0), z = VT(0);
           if (left > 0) x = __ldg(qx), y = __ldg(qy), z = __ldg(qz);
 #pragma unroll 1
@@ -269,7 +270,7 @@ __global__ void __launch_bounds__(32 * kGWarps, kGBlocksPerSm)
                                in ? fx_offset(fx_from_words(wz.x, wz.y, t2), U2) : 0, cell);
           }
           double f[kOwn];
-          group_transpose<G, int64_t>([&](int q) { return fx_fold<kM6>(S, q); }, f, sc, lane);
+          group_transpose<G, int64_t>([&](int q) { return fx_fold<kM6>(S, q, fold); }, f, sc, lane);
 #pragma unroll
           for (int k = 0; k < kOwn; ++k) val[k] = b0 == 0 ? f[k] : val[k] + f[k];
         }
@@ -293,7 +294,7 @@ __global__ void __launch_bounds__(32 * kGWarps, kGBlocksPerSm)
 #pragma unroll
       for (int k = 0; k < kOwn; ++k) {
         // inv_n 2^s: a normal double times a power of two, exact
-        const int s = fx ? fx_exponent(wq[k], cell) : 0;
+        const int s = fx ? fx_exponent(wq[k], cell, fold) : 0;
         out[k] = val[k] * __hiloint2double(__double2hiint(inv_n) + (n > 0 ? s * (1 << 20) : 0), __double2loint(inv_n));
       }
       const double u11 = __shfl_sync(0xffffffffu, out[0], gbase), u22 = __shfl_sync(0xffffffffu, out[1], gbase + 1),

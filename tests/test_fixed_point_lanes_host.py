@@ -11,7 +11,7 @@ from fractions import Fraction
 import numpy as np
 import pytest
 
-from test_fixed_point_host import ROOT, exact
+from test_fixed_point_host import PAIRS, ROOT, TRIPLES, exact
 
 HARNESS = r"""
 #include <cmath>
@@ -38,6 +38,7 @@ extern "C" int cell(const double *v, int n, const double *U, int lanes, double *
     Uf[d] = (uint64_t)fx_from_words((uint32_t)(fx_bits(U[d]) >> 32), (uint32_t)fx_bits(U[d]), top[d]);
   }
   bool over = false;
+  const int fold = fx_fold_bits((n + lanes - 1) / lanes);
   for (int q = 0; q < 26; ++q) out[q] = 0;
   for (int b0 = 0; b0 < n; b0 += lanes * kFxBlock) {
     double block[26] = {};
@@ -47,7 +48,7 @@ extern "C" int cell(const double *v, int n, const double *U, int lanes, double *
         FxSums<true> S;
         int cnt = 0;
         for (int i = b0 + l; i < n && i < b0 + lanes * kFxBlock; i += lanes) ++cnt;
-        S.clear(cnt);
+        S.clear(cnt, fold);
         int k = 0;
         for (int i = b0 + l; i < n && i < b0 + lanes * kFxBlock; i += lanes, ++k) {
           if (k == kFxMid) S.carry();
@@ -58,13 +59,13 @@ extern "C" int cell(const double *v, int n, const double *U, int lanes, double *
           }
           fx_accumulate<true>(S, c[0], c[1], c[2], g);
         }
-        for (int q = 0; q < 26; ++q) over |= __builtin_add_overflow(f[q], fx_fold<true>(S, q), &f[q]);
+        for (int q = 0; q < 26; ++q) over |= __builtin_add_overflow(f[q], fx_fold<true>(S, q, fold), &f[q]);
       }
       for (int q = 0; q < 26; ++q) block[q] += (double)f[q];
     }
     for (int q = 0; q < 26; ++q) out[q] += block[q];
   }
-  for (int q = 0; q < 26; ++q) out[q] = std::ldexp(out[q], fx_exponent(fx_weights(q), g));
+  for (int q = 0; q < 26; ++q) out[q] = std::ldexp(out[q], fx_exponent(fx_weights(q), g, fold));
   return over ? -1 : 1;
 }
 """
@@ -122,3 +123,35 @@ def test_terms_near_their_bounds(cell, kind, n, lanes):
     ref, mag = exact(v, U)
     for q in range(26):
         assert abs(Fraction(float(got[q])) - ref[q]) <= mag[q] * Fraction(1, 2**48), q
+
+
+def fp64_sums(v, U):
+    """The 26 sums in FP64 by eight lanes."""
+    c = v - U[:, None]
+    r2 = c[0] * c[0] + c[1] * c[1] + c[2] * c[2]
+    rows = ([c[i] * c[j] for i, j in PAIRS] + [c[i] * c[j] * c[k] for i, j, k in TRIPLES]
+            + [r2 * (c[i] * c[j]) for i, j in PAIRS] + [r2 * r2 * c[i] for i in range(3)] + [r2 * r2 * r2])
+    out = []
+    for r in rows:
+        lane = np.zeros(8)
+        for i in range(0, r.size, 8):
+            lane[:r[i:i + 8].size] += r[i:i + 8]
+        out.append(((lane[0] + lane[4]) + (lane[2] + lane[6])) + ((lane[1] + lane[5]) + (lane[3] + lane[7])))
+    return out
+
+
+@pytest.mark.parametrize("lanes", [8, 32])
+@pytest.mark.parametrize("n", [9, 16, 30, 50, 91])
+def test_no_further_off_than_fp64_sums(cell, n, lanes):
+    """Over Maxwellian cells and all slots, the root mean square of the errors (in units of
+    the sum of the terms' magnitudes) is no larger than that of FP64 sums of the same cells."""
+    rng = np.random.default_rng(n)
+    fixed, plain = [], []
+    for _ in range(30):
+        v = rng.standard_normal((3, n)) + np.array([[0.5], [0.0], [-0.2]])
+        ok, U, got = cell(v, lanes)
+        assert ok == 1
+        ref, mag = exact(v, U)
+        for errs, x in ((fixed, got), (plain, fp64_sums(v, U))):
+            errs.append([float((Fraction(float(x[q])) - ref[q]) / mag[q]) for q in range(26)])
+    assert np.sqrt(np.mean(np.square(fixed))) <= np.sqrt(np.mean(np.square(plain)))
