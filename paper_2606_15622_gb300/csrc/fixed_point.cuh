@@ -273,4 +273,20 @@ FPC_HD int fx_exponent(uint32_t w, const FxCell &c, int fold = kFxFold) {
          (int)(w >> 24) * c.er;
 }
 
+// Whether a cell's tails are too heavy for fixed point: n w_ii > 2^kFxTail u_ii
+// max u_jj over the sums.  A Maxwellian has 5 there; one particle far out makes
+// it up to n.  Rounding is relative to the largest term that the bounds allow,
+// so sums to which ordinary particles contribute beside such a particle (u_12
+// beside outliers in c_1 and c_2) lose digits: a thousand particles with
+// outliers of 30 to 1e6 sigma came out up to 5,000 times as far off as FP64
+// sums, cells below the limit (and those of up to 2^kFxTail particles, which
+// cannot pass it) within a few times.
+// Compared as logarithms, the doubles' high words (the fraction taken as it is:
+// up to 0.09 below); lu: fx_log of u_ii, lmax: the largest of the cell.
+constexpr int kFxTail = 4;
+FPC_HD int32_t fx_log(uint32_t hi_u, int e, int fold) { return (int32_t)hi_u + (2 * e + fold - kFxBits) * (1 << 20); }
+FPC_HD bool fx_heavy(uint32_t hi_w, uint32_t hi_u, uint32_t hi_n, int er, int32_t lmax) {
+  return ((int32_t)hi_w - (int32_t)hi_u) + ((int32_t)hi_n - lmax) > (kFxTail - er) * (1 << 20);
+}
+
 }  // namespace fpc

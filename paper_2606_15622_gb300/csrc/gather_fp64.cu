@@ -19,7 +19,8 @@
 //
 // A cell outside the fixed-point form's reach takes its sums in FP64: a
 // velocity that is not finite, a component whose spread is below 2^-5 of its
-// speed or that does not vary at all, a spread beyond 2^+-120, and cells of up
+// speed or that does not vary at all, a spread beyond 2^+-120, tails so heavy
+// that fixed point loses digits (fx_heavy; known after the sums), and cells of up
 // to eight particles (one round of the lanes; their systems can be so
 // ill-conditioned that every rounding shows).
 #include <cstdint>
@@ -234,7 +235,7 @@ __global__ void __launch_bounds__(32 * kGWarps, kGBlocksPerSm)
       const uint2 uw = v_words(U);
       const uint64_t Uf = fx_from_words(uw.x, uw.y, fx_exp(mh) + kFxHead + 1023);
       const unsigned okmask = __ballot_sync(0xffffffffu, fixed);
-      const bool fx = ((~okmask >> gbase) & (0xffffffffu >> (32 - G))) == 0u;  // the whole cell
+      bool fx = ((~okmask >> gbase) & (0xffffffffu >> (32 - G))) == 0u;  // the whole cell
       const int fold = fx_fold_bits((n + G - 1) / G);
       const FxCell cell = fx_cell(__shfl_sync(0xffffffffu, mh, gbase), __shfl_sync(0xffffffffu, mh, gbase + 1),
                                   __shfl_sync(0xffffffffu, mh, gbase + 2));
@@ -274,6 +275,16 @@ __global__ void __launch_bounds__(32 * kGWarps, kGBlocksPerSm)
 #pragma unroll
           for (int k = 0; k < kOwn; ++k) val[k] = b0 == 0 ? f[k] : val[k] + f[k];
         }
+      }
+      {  // heavy tails: lane i < 3 of the group owns u_ii (slots 0, 3, 5) and w_ii
+        const uint32_t hu = (uint32_t)__double2hiint(lg == 0 ? val[0] : val[1]);
+        const uint32_t hw = (uint32_t)__double2hiint(lg == 0 ? val[2] : val[3]);
+        const int32_t lu = fx_log(hu, lg == 0 ? cell.e[0] : lg == 1 ? cell.e[1] : cell.e[2], fold);
+        const int32_t lmax = max(__shfl_sync(0xffffffffu, lu, gbase),
+                                 max(__shfl_sync(0xffffffffu, lu, gbase + 1), __shfl_sync(0xffffffffu, lu, gbase + 2)));
+        const uint32_t hn = (2u * 1023u << 20) - (uint32_t)__double2hiint(inv_n);  // of n
+        const unsigned heavy = __ballot_sync(0xffffffffu, lg < 3 && fx_heavy(hw, hu, hn, cell.er, lmax));
+        fx = fx && ((heavy >> gbase) & 7u) == 0u;
       }
       if (!__all_sync(0xffffffffu, fx || n == 0)) {  // some cell of the task in FP64
         const double Ux = __shfl_sync(0xffffffffu, U, gbase), Uy = __shfl_sync(0xffffffffu, U, gbase + 1),

@@ -18,7 +18,7 @@ HARNESS = r"""
 #include "fixed_point.cuh"
 using namespace fpc;
 // the central sums of one cell by `lanes` lanes, as gather_fp64_kernel forms them; 0: refused,
-// -1: an integer sum overflowed
+// 2: its tails are too heavy, -1: an integer sum overflowed
 extern "C" int cell(const double *v, int n, const double *U, int lanes, double *out) {
   uint32_t mh[3];
   for (int d = 0; d < 3; ++d) {
@@ -65,7 +65,17 @@ extern "C" int cell(const double *v, int n, const double *U, int lanes, double *
     }
     for (int q = 0; q < 26; ++q) out[q] += block[q];
   }
+  const int u[3] = {0, 3, 5};
+  const auto hi = [](double x) { return (uint32_t)(fx_bits(x) >> 32); };
+  int32_t lmax = 0;
+  for (int d = 0; d < 3; ++d) {
+    const int32_t lu = fx_log(hi(out[u[d]]), g.e[d], fold);
+    lmax = lu > lmax ? lu : lmax;
+  }
+  bool heavy = false;
+  for (int d = 0; d < 3; ++d) heavy |= fx_heavy(hi(out[16 + u[d]]), hi(out[u[d]]), hi(n), g.er, lmax);
   for (int q = 0; q < 26; ++q) out[q] = std::ldexp(out[q], fx_exponent(fx_weights(q), g, fold));
+  if (heavy) return 2;
   return over ? -1 : 1;
 }
 """
@@ -155,3 +165,55 @@ def test_no_further_off_than_fp64_sums(cell, n, lanes):
         for errs, x in ((fixed, got), (plain, fp64_sums(v, U))):
             errs.append([float((Fraction(float(x[q])) - ref[q]) / mag[q]) for q in range(26)])
     assert np.sqrt(np.mean(np.square(fixed))) <= np.sqrt(np.mean(np.square(plain)))
+
+
+def heavy(kind, n, rng):
+    """Maxwellian cells with outliers in one or two components, hot tails, Student's t."""
+    v = rng.standard_normal((3, n))
+    if kind == "student":
+        return rng.standard_t(3, (3, n))
+    if kind == "hot tail":
+        v[:, rng.random(n) < 0.02] *= 6.5
+    else:
+        size, components = kind
+        for d in range(components):
+            v[d, d] = size * (1 + 0.1 * rng.random())
+    return v
+
+
+HEAVY = ["student", "hot tail"] + [(size, k) for size in (6, 10, 30, 1e3, 1e6) for k in (1, 2)]
+
+
+def bounds(mag, most, n):
+    """What a cell's sums may be off by: FP64 sums by eight lanes add n / 8 terms a lane and
+    round terms and lanes' sums some 16 times, 2^-53 of the terms' magnitudes `mag` each.
+    Cells of up to 16 particles are never taken for heavy, so there also the fixed-point
+    form's own part: up to 8 units of 2^-58 of the largest possible term a particle, whose
+    factors are bounded by powers of two (|c_d| < 2 max |c_d|, |c|^2 < 8 sum max c_d^2)."""
+    m = [2 * x for x in most]
+    r2 = 2 * sum(x * x for x in m)
+    top = ([m[i] * m[j] for i, j in PAIRS] + [m[i] * m[j] * m[k] for i, j, k in TRIPLES]
+           + [r2 * m[i] * m[j] for i, j in PAIRS] + [r2 * r2 * m[i] for i in range(3)] + [r2 * r2 * r2])
+    return [a * (n // 8 + 16) * 2.0**-53 + (n * t * 2.0**-55 if n <= 16 else 0.0) for a, t in zip(mag, top)]
+
+
+@pytest.mark.parametrize("lanes", [8, 32])
+@pytest.mark.parametrize("kind", HEAVY, ids=str)
+def test_heavy_tails(cell, kind, lanes):
+    """Cells that fixed point takes stay within `bounds`."""
+    rng = np.random.default_rng(1)
+    for n in (9, 16, 30, 100, 300, 1000):
+        v = heavy(kind, n, rng)
+        ok, U, got = cell(v, lanes)
+        assert ok in (1, 2)
+        if ok == 1:
+            ref, mag = exact(v, U)
+            for q, most in enumerate(bounds([float(x) for x in mag], np.abs(v - U[:, None]).max(1), n)):
+                assert abs(Fraction(float(got[q])) - ref[q]) <= most, (n, q)
+
+
+def test_maxwellian_cells_are_taken(cell):
+    rng = np.random.default_rng(2)
+    for n in (9, 12, 20, 50, 200):
+        for _ in range(200):
+            assert cell(rng.standard_normal((3, n)) * [[1.0], [2.0], [0.5]], 8)[0] == 1
