@@ -40,6 +40,7 @@ static_assert(kFxLanes * kFxBlock < 1 << (63 - kFxBits + kFxFold), "the folded b
 // is only ever shifted right)
 constexpr int kFxHead = 63 - kFxBits;
 constexpr int kFxMaxExp = 120;  // |E| accepted: 2^(5 E) and 2^(6 E) stay normal doubles
+constexpr int kFxMinExpF = -67;  // of FP32 velocities: their subnormals, read as zero, are below half a unit
 
 struct Fx {
   int32_t h, l;

@@ -19,9 +19,9 @@
 //
 // A cell outside the fixed-point form's reach takes its sums in FP64: a
 // velocity that is not finite, a component whose spread is below 2^-5 of its
-// speed or that does not vary at all, a spread beyond 2^+-120, tails so heavy
-// that fixed point loses digits (fx_heavy; known after the sums), and cells of up
-// to eight particles (one round of the lanes; their systems can be so
+// speed or that does not vary at all, a spread beyond 2^+-120 (FP32 velocities:
+// below 2^-67), tails so heavy that fixed point loses digits (fx_heavy; known
+// after the sums), and cells of up to eight particles (one round of the lanes; their systems can be so
 // ill-conditioned that every rounding shows).
 #include <cstdint>
 
@@ -53,7 +53,7 @@ __device__ __forceinline__ void accumulate26d(double (&t)[kNSum], double cx, dou
 }
 
 // a velocity as the two words of its double (FP32 values on the integer pipe;
-// FP32 subnormals, which the fixed point drops anyway, read as zero there)
+// FP32 subnormals read as zero there: see kFxMinExpF)
 __device__ __forceinline__ uint2 v_words(double x) {
   return make_uint2((uint32_t)__double2hiint(x), (uint32_t)__double2loint(x));
 }
@@ -231,7 +231,8 @@ __global__ void __launch_bounds__(32 * kGWarps, kGBlocksPerSm)
       const int32_t klo = group_scatter3<G>(lo0, lo1, lo2, 0, lg, [](int32_t p, int32_t q) { return min(p, q); });
       const int32_t khi = group_scatter3<G>(hi0, hi1, hi2, 0, lg, [](int32_t p, int32_t q) { return max(p, q); });
       uint32_t mh;
-      const bool fixed = (fx_range(U, klo, khi, mh) && n > kGFew) || (lg & 3) == 3;
+      const bool ranged = fx_range(U, klo, khi, mh) && (sizeof(VT) == 8 || fx_exp(mh) >= kFxMinExpF);
+      const bool fixed = (ranged && n > kGFew) || (lg & 3) == 3;
       const uint2 uw = v_words(U);
       const uint64_t Uf = fx_from_words(uw.x, uw.y, fx_exp(mh) + kFxHead + 1023);
       const unsigned okmask = __ballot_sync(0xffffffffu, fixed);
