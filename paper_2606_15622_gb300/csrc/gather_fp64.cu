@@ -170,7 +170,9 @@ __global__ void __launch_bounds__(32 * kGWarps, kGBlocksPerSm)
   auto share = [&](int64_t k) { return base0 + (total / nwarps) * k + (total % nwarps) * k / nwarps; };
   const int64_t Lx = lower_bound16_by([&](int64_t c) { return off[c] + kGCellWork * c; }, n_cells,
                                       share(lane < 16 ? warp : warp + 1), lane);
-  const int64_t ca = __shfl_sync(0xffffffffu, Lx, 0), cb = __shfl_sync(0xffffffffu, Lx, 16);
+  // (whole tasks: a share of nine cells would be three tasks of four, four and one)
+  const int64_t whole = min((Lx + kCells - 1) / kCells * kCells, n_cells);
+  const int64_t ca = __shfl_sync(0xffffffffu, whole, 0), cb = __shfl_sync(0xffffffffu, whole, 16);
   for (int64_t c0 = ca; c0 < cb; c0 += 32) {
     const int ncell = (int)(cb - c0 < 32 ? cb - c0 : 32);
     // rank the run's cells by size, largest first (bitonic; lane l's cell is
