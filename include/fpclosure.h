@@ -86,9 +86,9 @@ enum { FP_V_F32 = 0, FP_V_F64 = 1 };
  * b - A x, formed in pairs of FP32 numbers (~46 bits; agreeing with the FP64
  * elimination to ~1e-9 relative, far below the moments' own error); cells
  * whose FP32 pivots fall below max(3e-3, 100 pivot_rtol) of max|A|, whose
- * correction exceeds 1e-4 of the solution, or whose theta or tau lies beyond
- * 2^+-20, are eliminated in FP64 instead, and that elimination decides their
- * flags.  With FP32
+ * correction exceeds 1e-4 of the solution, or whose theta lies beyond 2^+-20,
+ * are eliminated in FP64 instead, and that elimination decides their flags.
+ * With FP32
  * moments (relative error ~1e-7) a pivot below ~1e-6 max|A| cannot be told
  * from zero, so that mode flags a cell singular when a pivot is
  * <= max(pivot_rtol, FP_FP32_PIVOT_FLOOR) * max|A|.  A cell of four

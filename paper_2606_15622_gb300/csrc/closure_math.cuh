@@ -589,7 +589,12 @@ __device__ __forceinline__ int closure_cell_mixed(const double *__restrict__ mc,
                                                   double (&y)[9], bool &todo) {
   todo = false;
   int fl = 0;
-  bool in_range;  // of f2_split: theta and tau within 2^+-20, so z (order 5) within 2^+-50 of one
+  // The right-hand side is proportional to 1 / tau and tau stands nowhere else:
+  // the system is solved for tau's mantissa ts in [1, 2) and y takes the power of
+  // two 2^-kt, exactly.
+  double ts;
+  int kt;
+  bool in_range;  // of f2_split: theta within 2^+-20, so z (order 5) within 2^+-50 of one; 2^-kt y is a normal double
   {
     bool fin = finite_d(tc) && positive_d(tc);
 #pragma unroll
@@ -598,8 +603,10 @@ __device__ __forceinline__ int closure_cell_mixed(const double *__restrict__ mc,
     if (mc[kN] < (double)prm.min_particles) fl |= FP_FLAG_FEW;
     if (!positive_d(mc[kTheta])) fl |= FP_FLAG_SINGULAR;
     if (!fl && mc[kN] < (double)prm.min_regular) fl |= FP_FLAG_SINGULAR;
-    auto near_one = [](double v) { return (((uint32_t)__double2hiint(v) >> 20) & 0x7ffu) - (1023u - 20u) < 40u; };
-    in_range = near_one(tc) && near_one(mc[kTheta]);
+    auto exponent = [](double v) { return (int)(((uint32_t)__double2hiint(v) >> 20) & 0x7ffu) - 1023; };
+    kt = exponent(tc);
+    ts = __hiloint2double((__double2hiint(tc) & 0xfffff) | 0x3ff00000, __double2loint(tc));
+    in_range = (unsigned)(exponent(mc[kTheta]) + 20) < 40u && (unsigned)(kt + 900) < 1800u;
   }
   if (fl) {
     linear_drift(tc, y);
@@ -615,7 +622,7 @@ __device__ __forceinline__ int closure_cell_mixed(const double *__restrict__ mc,
     for (int r = 0; r < 9; ++r)
 #pragma unroll
       for (int c = 0; c < 10; ++c) af[r][c] = 0.f;
-    assemble_emit(mf, d2f_rn(tc), d2f_rn(prm.eps2_hat), [&](int row, int col, float v) { af[row][col] = v; });
+    assemble_emit(mf, d2f_rn(ts), d2f_rn(prm.eps2_hat), [&](int row, int col, float v) { af[row][col] = v; });
   }
   uint32_t amax = 0;
 #pragma unroll
@@ -639,14 +646,14 @@ __device__ __forceinline__ int closure_cell_mixed(const double *__restrict__ mc,
   if (ok) {
     back_sub_f(af, rinv, x0);
     float rf[9], d[9];
-    residual_f2(mc, tc, prm.eps2_hat, x0, rf);
+    residual_f2(mc, ts, prm.eps2_hat, x0, rf);
     lu_apply_f(af, rinv, perm, rf, d);
     float dmax = 0.f, xmax = 0.f;
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
       dmax = fmaxf(dmax, fabsf(d[q]));
       xmax = fmaxf(xmax, fabsf(x0[q]));
-      y[q] = f2d_exact(x0[q]) + f2d_exact(d[q]);
+      y[q] = f2d_exact(x0[q], -kt) + f2d_exact(d[q], -kt);
     }
     ok = dmax <= 1e-4f * xmax;
 #pragma unroll
