@@ -675,9 +675,10 @@ __device__ __forceinline__ int closure_cell_mixed(const double *__restrict__ mc,
 // (FP64 instructions have a latency of about 64 cycles on this GPU, a
 // reciprocal by rcp_d about 400), roughly halved, which is what a short
 // fallback list waits for.  The reciprocal of each candidate pivot runs beside
-// the pivot search.  The solve runs even for a flagged cell (the warp must stay
-// converged for the shuffles) and its result is then discarded; valid =
-// false makes the group a passenger: no loads, results meaningless.
+// the pivot search.  The solve runs also for a flagged cell beside one that is
+// not (the warp must stay converged for the shuffles) and its result is then
+// discarded; valid = false makes the group a passenger: no loads, results
+// meaningless.
 __device__ __forceinline__ int closure_cell_group16(const double *__restrict__ mc, double tc, const SolveParams &prm,
                                                     bool valid, int r, double (&y)[9]) {
   constexpr unsigned kAll = 0xffffffffu;
@@ -692,63 +693,66 @@ __device__ __forceinline__ int closure_cell_group16(const double *__restrict__ m
   if (m[kN] < (double)prm.min_particles) fl |= FP_FLAG_FEW;
   if (!positive_d(m[kTheta])) fl |= FP_FLAG_SINGULAR;
   if (!fl && m[kN] < (double)prm.min_regular) fl |= FP_FLAG_SINGULAR;
-
-  double row[10];
-#pragma unroll
-  for (int col = 0; col < 10; ++col) row[col] = 0.0;
-  assemble_emit(m, tc, prm.eps2_hat, [&](int rr, int col, double v) {
-    if (rr == r) row[col] = v;
-  });
-  // max |A| over the group (rows 9.. are zero)
-  uint64_t amax = 0;
-#pragma unroll
-  for (int j = 0; j < 9; ++j) amax = max(amax, abs_bits(row[j]));
-#pragma unroll
-  for (int o = 8; o >= 1; o >>= 1) amax = max(amax, (uint64_t)__shfl_xor_sync(kAll, (unsigned long long)amax, o, 16));
-  const double amax_d = __longlong_as_double((long long)amax);
   int sfl = 0;
-  if (!(amax_d > 0.0) || !finite_d(amax_d)) sfl = FP_FLAG_SINGULAR;
-  const uint64_t thr = abs_bits(prm.pivot_rtol * amax_d);
-  double rinv[9];
 #pragma unroll
-  for (int K = 0; K < 9; ++K) {
-    const double inv_own = rcp_d(row[K]);  // this lane's candidate reciprocal, beside the search
-    // pivot: the largest |a_iK| over rows i >= K, the first such row on ties
-    // (key 0 for lanes that are not candidates)
-    const bool cand = r >= K && r < 9;
-    uint64_t key = cand ? ((abs_bits(row[K]) << 1) | 1ull) : 0ull;
-    int idx = r;
+  for (int q = 0; q < 9; ++q) y[q] = 0.0;
+  if (__any_sync(kAll, valid && !fl)) {  // (flagged cells alone: nothing to solve)
+    double row[10];
 #pragma unroll
-    for (int o = 8; o >= 1; o >>= 1) {
-      const uint64_t k2 = __shfl_xor_sync(kAll, (unsigned long long)key, o, 16);
-      const int i2 = __shfl_xor_sync(kAll, idx, o, 16);
-      if (k2 > key || (k2 == key && i2 < idx)) {
-        key = k2;
-        idx = i2;
+    for (int col = 0; col < 10; ++col) row[col] = 0.0;
+    assemble_emit(m, tc, prm.eps2_hat, [&](int rr, int col, double v) {
+      if (rr == r) row[col] = v;
+    });
+    // max |A| over the group (rows 9.. are zero)
+    uint64_t amax = 0;
+#pragma unroll
+    for (int j = 0; j < 9; ++j) amax = max(amax, abs_bits(row[j]));
+#pragma unroll
+    for (int o = 8; o >= 1; o >>= 1) amax = max(amax, (uint64_t)__shfl_xor_sync(kAll, (unsigned long long)amax, o, 16));
+    const double amax_d = __longlong_as_double((long long)amax);
+    if (!(amax_d > 0.0) || !finite_d(amax_d)) sfl = FP_FLAG_SINGULAR;
+    const uint64_t thr = abs_bits(prm.pivot_rtol * amax_d);
+    double rinv[9];
+#pragma unroll
+    for (int K = 0; K < 9; ++K) {
+      const double inv_own = rcp_d(row[K]);  // this lane's candidate reciprocal, beside the search
+      // pivot: the largest |a_iK| over rows i >= K, the first such row on ties
+      // (key 0 for lanes that are not candidates)
+      const bool cand = r >= K && r < 9;
+      uint64_t key = cand ? ((abs_bits(row[K]) << 1) | 1ull) : 0ull;
+      int idx = r;
+#pragma unroll
+      for (int o = 8; o >= 1; o >>= 1) {
+        const uint64_t k2 = __shfl_xor_sync(kAll, (unsigned long long)key, o, 16);
+        const int i2 = __shfl_xor_sync(kAll, idx, o, 16);
+        if (k2 > key || (k2 == key && i2 < idx)) {
+          key = k2;
+          idx = i2;
+        }
+      }
+      const int bi = idx;
+      if (!((key >> 1) > thr)) sfl = FP_FLAG_SINGULAR;
+      // rows K and bi trade places; every lane reads the pivot row (old row bi)
+      const int src = r == K ? bi : (r == bi ? K : r);
+      double piv[10];
+#pragma unroll
+      for (int j = K; j < 10; ++j) {
+        piv[j] = __shfl_sync(kAll, row[j], bi, 16);
+        row[j] = __shfl_sync(kAll, row[j], src, 16);
+      }
+      rinv[K] = __shfl_sync(kAll, inv_own, bi, 16);
+      if (r > K && r < 9) {
+        const double l = row[K] * rinv[K];
+#pragma unroll
+        for (int j = K + 1; j < 10; ++j) row[j] = fma(-l, piv[j], row[j]);
       }
     }
-    const int bi = idx;
-    if (!((key >> 1) > thr)) sfl = FP_FLAG_SINGULAR;
-    // rows K and bi trade places; every lane reads the pivot row (old row bi)
-    const int src = r == K ? bi : (r == bi ? K : r);
-    double piv[10];
+    double s = row[9];
 #pragma unroll
-    for (int j = K; j < 10; ++j) {
-      piv[j] = __shfl_sync(kAll, row[j], bi, 16);
-      row[j] = __shfl_sync(kAll, row[j], src, 16);
+    for (int k = 8; k >= 0; --k) {
+      y[k] = __shfl_sync(kAll, s * rinv[k], k, 16);
+      s = fma(-row[k], y[k], s);  // every row's sum at once; the rows above k go on to use it
     }
-    rinv[K] = __shfl_sync(kAll, inv_own, bi, 16);
-    if (r > K && r < 9) {
-      const double l = row[K] * rinv[K];
-#pragma unroll
-      for (int j = K + 1; j < 10; ++j) row[j] = fma(-l, piv[j], row[j]);
-    }
-  }
-  double s = row[9];
-#pragma unroll
-  for (int k = 8; k >= 0; --k) {
-    y[k] = __shfl_sync(kAll, s * rinv[k], k, 16);
-    s = fma(-row[k], y[k], s);  // every row's sum at once; the rows above k go on to use it
   }
   if (!fl) {
     fl = sfl;
