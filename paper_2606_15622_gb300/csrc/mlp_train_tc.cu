@@ -656,6 +656,17 @@ __global__ void sum_tiles_kernel(const float *__restrict__ parts, int ntiles, in
   if (adam.p) adam_update(adam, dst, s);
 }
 
+static int train_sm_count() {
+  static int n = 0;
+  if (!n) {
+    int dev = 0, k = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&k, cudaDevAttrMultiProcessorCount, dev);
+    n = k > 0 ? k : 152;
+  }
+  return n;
+}
+
 size_t mlp_backward_tc_ws(int64_t n) {
   const int64_t tiles = (n + kBR - 1) / kBR;
   return (size_t)tiles * (size_t)mlp_param_count() * sizeof(float);
@@ -691,7 +702,17 @@ int launch_mlp_backward_adam_tc(const MlpDev &net, const void *x, const void *h_
     mlp_backward_tc_kernel<<<(unsigned)tiles, kBT, kBSmem, st>>>(net, xb, hb, z_save, db, dout, n, np, parts);
   AdamParams a{};
   if (adam) a = *adam;
-  launch_after(sum_tiles_kernel, (unsigned)((np + 255) / 256), 256, 0, st, parts, (int)tiles, np, grads, a);
+  // The sum's blocks start early only where the backward pass's last wave (a
+  // tile an SM) leaves room for them at four an SM: on fewer free SMs they all
+  // crowd there and read the partial sums through those.  152 SMs, us a step:
+  // 12,000 rows (94 tiles) 55.5 early, 57.7 late; 16,384 rows (128) 71.8, 59.8;
+  // 19,456 (152) 78.4, 64.1; 25,000 (152 + 44) 112.6, 113.9; 38,912 (304) 181.7, 133.2.
+  const unsigned blocks = (unsigned)((np + 255) / 256);
+  const int64_t sms = train_sm_count(), last = (tiles - 1) % sms + 1;
+  if (blocks <= 4 * (sms - last))
+    launch_after(sum_tiles_kernel, blocks, 256, 0, st, parts, (int)tiles, np, grads, a);
+  else
+    sum_tiles_kernel<<<blocks, 256, 0, st>>>(parts, (int)tiles, np, grads, a);
   return 0;
 }
 
