@@ -84,23 +84,27 @@ __device__ __forceinline__ void store_comp<double>(double *p, int cls, const dou
     p[0] = x[0], p[1] = x[1], p[2] = x[2], p[3] = x[3];
 }
 
-// FP64 -> T for a table.  To FP32 on the integer pipe, to nearest even, values
-// below the smallest normal number to zero: the FP64 pipe takes 68 cycles a
-// conversion, this about 20 (values past FP32's range, which branch, aside).
+// FP64 -> T for a table, rounded to nearest even.  To FP32 on the integer pipe:
+// the FP64 pipe takes 68 cycles a conversion, this about 20.  Values beyond
+// FP32's normal range, zeros aside, are converted by the FP64 pipe.
 template <typename T>
 __device__ __forceinline__ T narrow(double x);
 template <>
 __device__ __forceinline__ double narrow<double>(double x) { return x; }
 template <>
 __device__ __forceinline__ float narrow<float>(double x) {
-  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t hi = (uint32_t)__double2hiint(x);
+  uint32_t lo = (uint32_t)__double2loint(x);
   const uint32_t a = hi & 0x7fffffffu;
+  const bool common = a - (897u << 20) < (253u << 20);  // 2^-126 .. 2^127
   // the top 23 fraction bits under the exponent less 896 (modulo 2^32)
   uint32_t u = __funnelshift_l(lo, hi, 3) - (896u << 23);
   u += ((lo & 0x1fffffffu) + 0x0fffffffu + (u & 1u)) >> 29;
-  u = (a < (897u << 20) ? 0u : u & 0x7fffffffu) | (hi & 0x80000000u);
-  float f = __uint_as_float(u);
-  if (__builtin_expect(a >= (1150u << 20), 0)) f = (float)x;
+  float f = __uint_as_float((common ? u & 0x7fffffffu : 0u) | (hi & 0x80000000u));
+  if (__builtin_expect(!common && (a | lo), 0)) {
+    asm volatile("" : "+r"(lo));  // a branch, not computed beside the common case
+    f = (float)__hiloint2double((int)hi, (int)lo);
+  }
   return f;
 }
 
