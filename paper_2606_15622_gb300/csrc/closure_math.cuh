@@ -345,6 +345,8 @@ __device__ __forceinline__ int closure_cell(const double *__restrict__ mc, doubl
 // ---------------------------------------------------------------------------
 // A number as h + l, |l| about 2^-24 |h|: pairs of FP32 carry some 46 bits,
 // the residual of a solution whose own error is 2^-24 kappa needs about 40.
+// (Products whose rounding error is taken are __fmul_rn: contracted into a sum
+// that follows, the sum would hold the unrounded product.)
 struct F2 {
   float h, l;
 };
@@ -385,29 +387,30 @@ __device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
   return f2_fast(s, e + (a.l + b.l));
 }
 __device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
-  const float p = a.h * b.h;
+  const float p = __fmul_rn(a.h, b.h);
   return f2_fast(p, fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p))));
 }
 __device__ __forceinline__ F2 f2_mul(F2 a, float b) {
-  const float p = a.h * b;
+  const float p = __fmul_rn(a.h, b);
   return f2_fast(p, fmaf(a.l, b, fmaf(a.h, b, -p)));
 }
 __device__ __forceinline__ F2 f2_scale(F2 a, float b) { return F2{a.h * b, a.l * b}; }  // b a power of two
 __device__ __forceinline__ F2 f2_recip(F2 a) {  // one Newton step from 1 / h
   const float y = 1.f / a.h;
   const float e = fmaf(-a.l, y, fmaf(-a.h, y, 1.f));
-  return f2_fast(y, y * e);
+  const float s = fmaf(y, e, y);
+  return F2{s, fmaf(y, e, y - s)};
 }
 // (h, l) += a b without renormalising: h by two-sum, the rest into l
 __device__ __forceinline__ void f2_mac(F2 &s, F2 a, float b) {
-  const float p = a.h * b, e = fmaf(a.l, b, fmaf(a.h, b, -p));
+  const float p = __fmul_rn(a.h, b), e = fmaf(a.l, b, fmaf(a.h, b, -p));
   float t, f;
   two_sum(s.h, p, t, f);
   s.h = t;
   s.l += e + f;
 }
 __device__ __forceinline__ void f2_mac(F2 &s, F2 a, F2 b) {
-  const float p = a.h * b.h, e = fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p)));
+  const float p = __fmul_rn(a.h, b.h), e = fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p)));
   float t, f;
   two_sum(s.h, p, t, f);
   s.h = t;
