@@ -41,7 +41,14 @@ __device__ __forceinline__ double tmad(double a, double b, double c) { return fm
 __device__ __forceinline__ float tmad(float a, float b, float c) { return a * b + c; }
 __device__ __forceinline__ double trcp(double a) { return rcp_d(a); }
 __device__ __forceinline__ float trcp(float a) { return 1.f / a; }
-__device__ __forceinline__ double tquot(double a, double b) { return a * rcp_d(b); }
+// (a denominator whose reciprocal is not a normal number: the quotient may be one)
+__device__ __forceinline__ double tquot(double a, double b) {
+  if (__builtin_expect((((uint32_t)__double2hiint(b) >> 20) & 0x7ffu) - 1u >= 2044u, 0)) {
+    asm volatile("" : "+d"(b));  // a branch, not computed beside the common case
+    return a / b;
+  }
+  return a * rcp_d(b);
+}
 __device__ __forceinline__ float tquot(float a, float b) { return a / b; }
 
 struct SolveParams {
