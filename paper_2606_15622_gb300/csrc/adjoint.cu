@@ -231,22 +231,52 @@ __global__ void __launch_bounds__(128, kLU ? 3 : 2) adjoint_cell_kernel(const do
 // ---------------------------------------------------------------------------
 // particle gradient
 // ---------------------------------------------------------------------------
-constexpr int kAConst = 40;         // table entries per cell
+template <typename T>
+constexpr int kAConst = sizeof(T) == 4 ? 44 : 40;  // table entries per cell
 constexpr int64_t kACellWork = 50;  // a cell's share of building a chunk's table, in particles (24: 98 us, 100: 98, 50: 94)
 
-// Per-cell table of the particle polynomial, every coefficient already
-// divided by N and with its multiplicity.  With c = v - U, r2 = |c|^2 and
+// Per-cell table of the particle polynomial, every coefficient with its
+// multiplicity.  With c = v - U, r2 = |c|^2 and
 //   s_d = W_d . c + r2 z_d,    t = c . s + 3 r2 (z . c)
-//   dL/dv_d = B_d + sum_j c_j (Mu_dj + sum_{k >= j} A_{d,jk} c_k) + c_d t + r2 s_d
+//   N dL/dv_d = B_d + sum_j c_j (Mu_dj + sum_{k >= j} A_{d,jk} c_k) + c_d t + r2 s_d
 // (Mu from gm_u and gm_theta, A from gm_u3, W from gm_w, z from gm_z;
-// B = gm_U / N minus the cell mean of the rest).
-enum { AA3 = 0, AW = 18, AZ = 24, AMU = 28, AU = 34, AB = 37 };
+// B = gm_U minus the cell mean of the rest).  In nearly singular cells these terms
+// cancel to a thousandth and less, so in FP32 what each of them loses shows:
+//   - U is a pair (v - U rounded at |U| would be off by that over |c|);
+//   - the division by N comes last, not into every coefficient;
+//   - B, a sum of 27 products a component, is summed with its rounding errors.
+// (Each cell's gradient against 64 bits, the worst cells of eight cylinder
+// populations: 5.4e-7 in the geometric mean, 8.3e-7 with none of the three, 7.4e-7
+// without the pair.)  In FP64 the coefficients are divided by N.
+enum { AA3 = 0, AW = 18, AZ = 24, AMU = 28, AU = 34, AB = 37, AUL = 40, AIN = 43 };
+
+// a sum of products, in FP32 with its rounding errors
+template <typename T>
+struct ProductSum {
+  T h;
+  __device__ __forceinline__ void mac(T a, T b) { h = tfma(a, b, h); }
+  __device__ __forceinline__ T value() const { return h; }
+};
+template <>
+struct ProductSum<float> {
+  float h, l = 0.f;
+  __device__ __forceinline__ void mac(float a, float b) {
+    const float t = fmaf(a, b, h);
+    l += fmaf(a, b, h - t);  // (exact where |a b| <= |h|; two-sum: 3 us more, the same errors)
+    h = t;
+  }
+  __device__ __forceinline__ float value() const { return h + l; }
+};
 
 // One cell's table row by one lane, from its moment gradients (first half)
 // and its moments (second half) staged in T.
 template <typename T>
 struct ParticleRow {
-  T inv_n, Mu[6], B[3];
+  T inv_n, Mu[6];
+  ProductSum<T> B[3];
+
+  // over N, in FP64
+  __device__ __forceinline__ T part(T x) const { return sizeof(T) == 4 ? x : x * inv_n; }
 
   __device__ __forceinline__ void gradients(const T *gc, int n, T *row) {
     inv_n = n > 0 ? T(1) / T(n) : T(0);
@@ -258,56 +288,83 @@ struct ParticleRow {
       for (int j = 0; j < 3; ++j)
 #pragma unroll
         for (int k = j; k < 3; ++k)
-          r[AA3 + 6 * d + sym2(j, k)] = T(1 + (j == d) + (k == d)) * (gc[kU3 + sym3(d, j, k)] * inv_n);
+          r[AA3 + 6 * d + sym2(j, k)] = T(1 + (j == d) + (k == d)) * part(gc[kU3 + sym3(d, j, k)]);
 #pragma unroll
     for (int s = 0; s < 6; ++s) {
       const bool diag = s == 0 || s == 3 || s == 5;
-      r[AW + s] = (diag ? T(2) : T(1)) * (gc[kW + s] * inv_n);
+      r[AW + s] = (diag ? T(2) : T(1)) * part(gc[kW + s]);
     }
 #pragma unroll
-    for (int d = 0; d < 3; ++d) r[AZ + d] = gc[kZ + d] * inv_n;
+    for (int d = 0; d < 3; ++d) r[AZ + d] = part(gc[kZ + d]);
     r[27] = T(0);
     store_row(row, r);
-    const T gth = gc[kTheta] * inv_n * T(2.0 / 3.0);
+    const T gth = part(gc[kTheta]) * T(2.0 / 3.0);
 #pragma unroll
     for (int s = 0; s < 6; ++s) {
       const bool diag = s == 0 || s == 3 || s == 5;
-      Mu[s] = diag ? tfma(T(2), gc[kU2 + s] * inv_n, gth) : gc[kU2 + s] * inv_n;
+      Mu[s] = diag ? tfma(T(2), part(gc[kU2 + s]), gth) : part(gc[kU2 + s]);
     }
 #pragma unroll
-    for (int d = 0; d < 3; ++d) B[d] = gc[kU + d] * inv_n;
+    for (int d = 0; d < 3; ++d) B[d].h = part(gc[kU + d]);
   }
 
-  // B less the cell mean of the polynomial, from the moments
-  __device__ __forceinline__ void moments(const T *mc, T *row) {
-    T u3[10], b[3];
+  // B less the cell mean of the polynomial, from the moments; U: the means in FP64
+  __device__ __forceinline__ void moments(const T *mc, const double *U, T *row) {
+    T u3[10];
 #pragma unroll
     for (int s = 0; s < 10; ++s) u3[s] = mc[kU3 + s];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) b[i] = u3[sym3(i, 0, 0)] + u3[sym3(i, 1, 1)] + u3[sym3(i, 2, 2)];
-    T s4 = T(0);
 #pragma unroll
     for (int j = 0; j < 3; ++j)
 #pragma unroll
       for (int k = j; k < 3; ++k) {
         const T u = mc[kU2 + sym2(j, k)], w = mc[kW + sym2(j, k)];
         const T Wjk = row[AW + sym2(j, k)] * (j == k ? T(1) : T(2));
-        if (j == k) s4 += w;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-          B[d] = tfma(-row[AA3 + 6 * d + sym2(j, k)], u, B[d]);
-          B[d] = tfma(-Wjk, u3[sym3(d, j, k)], B[d]);
+          B[d].mac(-row[AA3 + 6 * d + sym2(j, k)], u);
+          B[d].mac(-Wjk, u3[sym3(d, j, k)]);
         }
-        B[j] = tfma(T(-4) * row[AZ + k], w, B[j]);
-        if (j != k) B[k] = tfma(T(-4) * row[AZ + j], w, B[k]);
+        B[j].mac(T(-4) * row[AZ + k], w);
+        if (j != k) B[k].mac(T(-4) * row[AZ + j], w);
       }
+    if constexpr (sizeof(T) == 4) {
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
+      for (int d = 0; d < 3; ++d)
 #pragma unroll
-      for (int j = 0; j < 3; ++j) B[d] = tfma(-row[AW + sym2(d, j)], b[j], B[d]);
-      B[d] = tfma(-s4, row[AZ + d], B[d]);
+        for (int j = 0; j < 3; ++j) {
+          B[d].mac(-row[AZ + d], mc[kW + sym2(j, j)]);
+#pragma unroll
+          for (int k = 0; k < 3; ++k) B[d].mac(-row[AW + sym2(d, j)], u3[sym3(j, k, k)]);
+        }
+    } else {  // (fewer operations: the sums over k, and of the w_kk, first)
+      const T s4 = mc[kW] + mc[kW + 3] + mc[kW + 5];
+      T b[3];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) b[i] = u3[sym3(i, 0, 0)] + u3[sym3(i, 1, 1)] + u3[sym3(i, 2, 2)];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) B[d].mac(-row[AW + sym2(d, j)], b[j]);
+        B[d].mac(-s4, row[AZ + d]);
+      }
     }
-    const T r[12] = {Mu[0], Mu[1], Mu[2], Mu[3], Mu[4], Mu[5], mc[kU], mc[kU + 1], mc[kU + 2], B[0], B[1], B[2]};
+    T u[3] = {mc[kU], mc[kU + 1], mc[kU + 2]};
+    if constexpr (sizeof(T) == 4) {
+      float r[4];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const double x = U[d];
+        r[d] = 0.f;
+        if ((((uint32_t)__double2hiint(x) >> 20) & 0x7ffu) - (1023u - 100u) < 200u) {  // of f2_split
+          const F2 s = f2_split(x);
+          u[d] = s.h;
+          r[d] = s.l;
+        }
+      }
+      r[3] = inv_n;
+      store_row(row + AUL, r);
+    }
+    const T r[12] = {Mu[0], Mu[1], Mu[2], Mu[3], Mu[4], Mu[5], u[0], u[1], u[2], B[0].value(), B[1].value(), B[2].value()};
     store_row(row + AMU, r);
   }
 };
@@ -319,8 +376,8 @@ struct ParticleRow {
 // alignment allows, the next quad loaded while one is computed, and one table
 // row loaded a quad (another where a quad crosses a cell).  Bound: FP32 by the
 // loads in flight and the tables' building (11.9M particles of 131,072 cells
-// 114 us with a 44-entry row and three 4-byte loads a particle, 83 now; 288 MB
-// at the copy rate: 42); FP64 by its pipe, 59 operations a particle (75
+// 114 us with eight lanes a cell and three 4-byte loads a particle, 90 now, 83
+// without the terms that hold its error down; 288 MB at the copy rate: 42); FP64 by its pipe, 59 operations a particle (75
 // before, and the table was built eight lanes a cell): 819,200 particles
 // 212 -> 107 us (the operations alone: 96).  Registers: FP32 96 or 168 a
 // thread 102 / 92 us, FP64 168 a thread 112.
@@ -395,7 +452,7 @@ __global__ void __launch_bounds__(sizeof(VT) == 4 ? 128 : 64, 4)
         stage_rows<FP_NMOM>(mom + cbase * FP_NMOM, ncell, stage, lane);
         __syncwarp();
       }
-      if (valid) r.moments(stage + (lane + (both ? 16 : 0)) * kIn, tab + lane * kRow);
+      if (valid) r.moments(stage + (lane + (both ? 16 : 0)) * kIn, mom + c * FP_NMOM + kU, tab + lane * kRow);
     }
     __syncwarp();
     for (; qb < qe; qb += 128) {
@@ -414,7 +471,7 @@ __global__ void __launch_bounds__(sizeof(VT) == 4 ? 128 : 64, 4)
 #pragma unroll
       for (int st = 16; st >= 1; st >>= 1)
         if (co[cl + st] <= q0) cl += st;
-      T K[kAConst];
+      T K[kAConst<T>];
       load_row(tab + cl * kRow, K);
       int next = cl < 31 ? co[cl + 1] : INT_MAX;  // where the next cell starts
 #pragma unroll
@@ -426,7 +483,11 @@ __global__ void __launch_bounds__(sizeof(VT) == 4 ? 128 : 64, 4)
           load_row(tab + cl * kRow, K);
           next = cl < 31 ? co[cl + 1] : INT_MAX;
         }
-        const T cc[3] = {mx[u] - K[AU], my[u] - K[AU + 1], mz[u] - K[AU + 2]};
+        T cc[3] = {mx[u] - K[AU], my[u] - K[AU + 1], mz[u] - K[AU + 2]};
+        if constexpr (sizeof(T) == 4) {
+#pragma unroll
+          for (int d = 0; d < 3; ++d) cc[d] -= K[AUL + d];
+        }
         const T r2 = tfma(cc[0], cc[0], tfma(cc[1], cc[1], cc[2] * cc[2]));
         T s[3], out[3];
 #pragma unroll
@@ -448,6 +509,7 @@ __global__ void __launch_bounds__(sizeof(VT) == 4 ? 128 : 64, 4)
             g = tfma(cc[j], h, g);
           }
           out[d] = tfma(r2, s[d], tfma(cc[d], t, g));
+          if constexpr (sizeof(T) == 4) out[d] *= K[AIN];
         }
         mx[u] = out[0];
         my[u] = out[1];
