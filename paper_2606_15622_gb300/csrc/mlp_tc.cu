@@ -280,7 +280,7 @@ __device__ __forceinline__ void stage_source(const FusedIO &io, int64_t r0, int6
     for (int k = 0; k < kAt; ++k) {
       const int i = (k0 + k) * kT + t, r = i / kS, q = i - r * kS;
       float f;
-      if (__builtin_expect(!narrow_common(x[k], f) || (q == kTheta && f < 0.f), 0)) {
+      if (__builtin_expect((!narrow_common(x[k], f) || (q == kTheta && f < 0.f)) && i < total, 0)) {
         f = narrow(x[k]);
         if (!finite_d(x[k])) atomicOr(&pre[r], FP_FLAG_NONFINITE);
         if (q == kTheta && !positive_d(x[k])) atomicOr(&pre[r], FP_FLAG_SINGULAR);
