@@ -226,6 +226,7 @@ __global__ void __launch_bounds__(128, kLU ? 2 : 3) solve_kernel(const double *_
 // thread's in half the time, and one late cell does not hold up its warp for
 // a whole single-lane elimination (25 us).  Out of line: its registers are not
 // the mixed path's.
+template <bool kSkip = false>
 static __device__ __noinline__ void solve_listed(unsigned todo, int64_t c0, const double *__restrict__ mom,
                                                  const double *__restrict__ tau, const SolveParams &prm,
                                                  double *__restrict__ coeffs, int32_t *__restrict__ flags) {
@@ -239,7 +240,7 @@ static __device__ __noinline__ void solve_listed(unsigned todo, int64_t c0, cons
     const bool valid = mine >= 0;
     const int64_t c = c0 + (valid ? mine : first);
     double y[9];
-    const int fl = closure_cell_group16(mom + c * FP_NMOM, tau[c], prm, valid, r, y);
+    const int fl = closure_cell_group16<kSkip>(mom + c * FP_NMOM, tau[c], prm, valid, r, y);
     if (valid && r == 0) {
 #pragma unroll
       for (int q = 0; q < 9; ++q) coeffs[c * 9 + q] = y[q];
@@ -328,7 +329,7 @@ __global__ void __launch_bounds__(128) solve_group_kernel(const double *__restri
                                                           SolveParams prm, double *__restrict__ coeffs,
                                                           int32_t *__restrict__ flags) {
   const int64_t c0 = 2 * (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  if (c0 < n_cells) solve_listed(c0 + 1 < n_cells ? 3u : 1u, c0, mom, tau, prm, coeffs, flags);
+  if (c0 < n_cells) solve_listed<true>(c0 + 1 < n_cells ? 3u : 1u, c0, mom, tau, prm, coeffs, flags);
 }
 
 // ---------------------------------------------------------------------------

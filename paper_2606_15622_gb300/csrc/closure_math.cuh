@@ -685,10 +685,12 @@ __device__ __forceinline__ int closure_cell_mixed(const double *__restrict__ mc,
 // (FP64 instructions have a latency of about 64 cycles on this GPU, a
 // reciprocal by rcp_d about 400), roughly halved, which is what a short
 // fallback list waits for.  The reciprocal of each candidate pivot runs beside
-// the pivot search.  The solve runs also for a flagged cell beside one that is
-// not (the warp must stay converged for the shuffles) and its result is then
-// discarded; valid = false makes the group a passenger: no loads, results
-// meaningless.
+// the pivot search.  The solve runs also for a flagged cell (the warp must stay
+// converged for the shuffles) and its result is then discarded; with kSkip a warp
+// whose cells are both flagged solves nothing (lists of cells that need the solve
+// do without the question).  valid = false makes the group a passenger: no loads,
+// results meaningless.
+template <bool kSkip = false>
 __device__ __forceinline__ int closure_cell_group16(const double *__restrict__ mc, double tc, const SolveParams &prm,
                                                     bool valid, int r, double (&y)[9]) {
   constexpr unsigned kAll = 0xffffffffu;
@@ -704,9 +706,11 @@ __device__ __forceinline__ int closure_cell_group16(const double *__restrict__ m
   if (!positive_d(m[kTheta])) fl |= FP_FLAG_SINGULAR;
   if (!fl && m[kN] < (double)prm.min_regular) fl |= FP_FLAG_SINGULAR;
   int sfl = 0;
+  if (kSkip) {
 #pragma unroll
-  for (int q = 0; q < 9; ++q) y[q] = 0.0;
-  if (__any_sync(kAll, valid && !fl)) {  // (flagged cells alone: nothing to solve)
+    for (int q = 0; q < 9; ++q) y[q] = 0.0;
+  }
+  if (!kSkip || __any_sync(kAll, valid && !fl)) {
     double row[10];
 #pragma unroll
     for (int col = 0; col < 10; ++col) row[col] = 0.0;
