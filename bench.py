@@ -45,8 +45,8 @@ METRIC = "closure cells/s + particles/s (exact FP64, FP32-moment, surrogate) at 
 L2_FLUSH_BYTES = 256 << 20
 # DRAM bytes (read + write) of one launch in the ncu captures summarised under
 # profiles/ (current kernels; a kernel changed since its capture has none)
-NCU_DRAM_BYTES = {"velocity_update": 298.03e6, "gather_fp32": 175.77e6, "solve_mixed": 34.37e6,
-                  "gather_fp64": 326.46e6}
+NCU_DRAM_BYTES = {"velocity_update": 298.03e6, "gather_fp32": 175.77e6, "solve_mixed": 34.53e6,
+                  "gather_fp64": 326.24e6}
 ORACLE_BLOCK = 4096            # cells per block of the CPU oracle's timing
 E2E_CHUNKS = 8                 # chunks of the host-resident step (copy / compute overlap)
 WEIGHTS = os.path.join(ROOT, "paper_2606_15622_gb300", "weights", "surrogate_full.fpw")

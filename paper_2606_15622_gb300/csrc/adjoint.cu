@@ -561,10 +561,6 @@ __host__ __device__ constexpr int mult3(int s) { return (s == 0 || s == 6 || s =
 // 8-lane group folds its cell's moments and moment gradients into the 35
 // coefficients of the per-particle polynomial (shared-memory table), then all
 // 32 lanes walk the four cells' contiguous particle range.
-// A warp takes four consecutive cells; an 8-lane group folds its cell's
-// moments and moment gradients into the 35 coefficients of the per-particle
-// polynomial (shared-memory table), then all 32 lanes walk the four cells'
-// contiguous particle range.
 __global__ void __launch_bounds__(32 * kAWarps, 3)
     adjoint_particle_group_kernel(const float *__restrict__ v, int64_t np, const int64_t *__restrict__ off,
                                   int64_t n_cells, const double *__restrict__ mom, const double *__restrict__ gm,
@@ -738,8 +734,10 @@ static int adj_sm_count() {
 // FP32 calls on up to this many cells take the group kernel: a table of four
 // cells by eight lanes each is ready sooner than one of 32 by a lane each, and
 // its small footprint runs beside other streams' kernels (16,384 cells of 50
-// particles 11.9 us against 12.4, of 150 25.3 against 19.8; as a chunk of the
-// host-resident step 26.6 against 31; 40,000 cells of 50: 25.0 against 24.1)
+// particles 11.9 us against 12.4; as a chunk of the host-resident step 26.6
+// against 31; 40,000 cells of 50: 25.0 against 24.1).  The line is drawn by cells
+// alone: with more particles a cell the other kernel is ahead below it already
+// (16,384 cells of 150: 25.3 here, 19.8 there).
 constexpr int64_t kGroupCells = 32768;
 
 // A persistent grid (fewer blocks for small problems: two cells a warp at

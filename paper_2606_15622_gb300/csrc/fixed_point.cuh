@@ -1,18 +1,22 @@
 // fixed_point.cuh -- the fixed-point arithmetic of the FP64 moment gather.
 //
 // GB300 issues one FP64 warp instruction every 64 cycles per SM sub-partition
-// (68 measured) but one 32 x 32 + 64-bit integer multiply-add every 2, so the
-// 26 central sums of a cell (61 FP64 flops a particle) are formed in integers:
-// a component of c = v - U is an integer in units of 2^(E - 58), E the
+// (68 measured) but one 32 x 32 + 64-bit integer multiply-add every 4 to 6, so
+// the 26 central sums of a cell (61 FP64 flops a particle) are formed in
+// integers: a component of c = v - U is an integer in units of 2^(E - 58), E the
 // exponent with |c| < 2^E over the cell, held as two limbs h 2^29 + l,
 // 0 <= l < 2^29.  A product that is only summed takes three multiply-adds into
 // two 64-bit sums (h h', h l' + l h'); the dropped l l' is below 2^-58 of the
-// largest product, where an FP64 product is rounded at 2^-53 of itself
-// (<|c|^6> keeps it, the others its mean).  A product that is a factor
-// again (c_i c_j, |c|^2, |c|^4) is rounded to 2^-58 of its largest value.
+// largest product (<|c|^6> keeps it, the others its mean).  A product that is a
+// factor again (c_i c_j, |c|^2, |c|^4) is rounded to 2^-58 of its largest value.
 // Every component has its own exponent, and so has |c|^2 (the least power of
 // two above the sum of the components' squared bounds), so a thin
 // distribution keeps its digits.
+//
+// So a term is not exact but off by up to some 8 units of 2^-58 of the largest
+// term that the bounds allow, where an FP64 term is rounded at 2^-53 of itself:
+// closer than FP64 sums for Maxwellians, uniform cubes, beams and shock mixtures,
+// less close where few particles lie far outside the others, which fx_heavy finds.
 //
 // Plain C++ but for the qualifiers: the host test compiles it with g++.
 #pragma once

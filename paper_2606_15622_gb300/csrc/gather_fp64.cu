@@ -12,7 +12,8 @@
 // from L1 / L2.  What bounds it: instruction issue on the integer pipes, whose
 // 32 x 32-bit wide products (74 a particle) issue every 4 to 6 cycles; the
 // same sums on the FP64 pipe take 41 instructions of 68 cycles each.  On
-// 131,072 cells of 11.9M particles: 0.41 ms, where FP64 sums took 1.75 ms.
+// 131,072 cells of 11.9M particles: 0.41 ms, where FP64 sums took 1.75 ms (and
+// still do where every cell takes them).
 // Every warp of a resident grid takes an equal share of the work and walks its
 // cells in runs of up to 32, ranked by size so that the four cells of a task
 // have similar trip counts.
@@ -348,7 +349,7 @@ template <typename VT>
 static void launch_t(const VT *v, int64_t np, const int64_t *off, int64_t n_cells, double *mom, double *m6,
                      cudaStream_t st, int sm_count) {
   // a whole warp a cell while every cell has a resident warp of its own (the
-  // time is one cell's chain then: 400 cells of 100 particles 9.3 us, 14.5
+  // time is one cell's chain then: 400 cells of 100 particles 9.7 us, 14.5
   // with eight lanes); beyond, eight lanes (16: 461 us against 411 on 131,072
   // cells of 91 particles, 4: 510)
   if (n_cells <= (int64_t)sm_count * kGBlocksPerSm * kGWarps)
