@@ -11,6 +11,8 @@
 namespace fpc {
 void launch_gather(const void *v, int v_dtype, int64_t np, const int64_t *off, int64_t n_cells, int prec,
                    double *mom, double *m6, cudaStream_t st);
+void launch_gather_part(const void *v, int v_dtype, int64_t np, const int64_t *off, int64_t n_cells, int64_t whole,
+                        int prec, double *mom, double *m6, cudaStream_t st);
 void launch_solve(const double *mom, const double *tau, int64_t n_cells, const fp_params &p, int prec,
                   double *coeffs, int32_t *flags, double *lu, cudaStream_t st);
 void launch_velocity(const void *v, void *v_out, int v_dtype, int64_t np, const int64_t *off, int64_t n_cells,
@@ -116,6 +118,23 @@ namespace fpc {
 int report(int code, const char *msg) { return fail(code, "%s", msg); }
 }  // namespace fpc
 
+// fp_moments of n_cells that are a part of a call of `whole` cells (fp_step_host's chunks)
+namespace fpc {
+int moments_of_part(const void *v, int v_dtype, int64_t n_particles, const int64_t *cell_offsets, int64_t n_cells,
+                    int64_t whole, int prec, double *moments_out, double *m6_out, fp_stream_t stream) {
+  g_err[0] = 0;
+  if (n_cells < 0 || n_particles < 0) return fail(FP_ERR_ARG, "negative size");
+  if (n_cells == 0) return FP_OK;
+  if (v_dtype != FP_V_F32 && v_dtype != FP_V_F64) return fail(FP_ERR_ARG, "v_dtype %d", v_dtype);
+  if (prec != FP_PREC_FP64 && prec != FP_PREC_FP32_MOMENTS) return fail(FP_ERR_ARG, "prec %d", prec);
+  if (!cell_offsets || !moments_out) return fail(FP_ERR_ARG, "null array pointer");
+  if (n_particles > 0 && !v) return fail(FP_ERR_ARG, "null velocity pointer");
+  launch_gather_part(v, v_dtype, n_particles, cell_offsets, n_cells, whole, prec, moments_out, m6_out,
+                     (cudaStream_t)stream);
+  return check_launch("gather");
+}
+}  // namespace fpc
+
 extern "C" {
 
 void fp_default_params(fp_params *p) {
@@ -181,16 +200,8 @@ int fp_closure_exact(const void *v, int v_dtype, int64_t n_particles, const int6
 
 int fp_moments(const void *v, int v_dtype, int64_t n_particles, const int64_t *cell_offsets, int64_t n_cells,
                int prec, double *moments_out, double *m6_out, fp_stream_t stream) {
-  g_err[0] = 0;
-  if (n_cells < 0 || n_particles < 0) return fail(FP_ERR_ARG, "negative size");
-  if (n_cells == 0) return FP_OK;
-  if (v_dtype != FP_V_F32 && v_dtype != FP_V_F64) return fail(FP_ERR_ARG, "v_dtype %d", v_dtype);
-  if (prec != FP_PREC_FP64 && prec != FP_PREC_FP32_MOMENTS) return fail(FP_ERR_ARG, "prec %d", prec);
-  if (!cell_offsets || !moments_out) return fail(FP_ERR_ARG, "null array pointer");
-  if (n_particles > 0 && !v) return fail(FP_ERR_ARG, "null velocity pointer");
-  fpc::launch_gather(v, v_dtype, n_particles, cell_offsets, n_cells, prec, moments_out, m6_out,
-                     (cudaStream_t)stream);
-  return check_launch("gather");
+  return fpc::moments_of_part(v, v_dtype, n_particles, cell_offsets, n_cells, n_cells, prec, moments_out, m6_out,
+                              stream);
 }
 
 int fp_closure_solve(const double *moments, const double *tau, int64_t n_cells, const fp_params *p, int prec,

@@ -363,17 +363,23 @@ static void launch_gather_fp32(const void *v, int v_dtype, int64_t np, const int
 
 bool launch_gather_tile(const float *v, int64_t np, const int64_t *off, int64_t n_cells, double *mom, double *m6,
                         cudaStream_t st, int sm_count);
-void launch_gather_fp64(const void *v, int v_dtype, int64_t np, const int64_t *off, int64_t n_cells, double *mom,
-                        double *m6, cudaStream_t st, int sm_count);
+void launch_gather_fp64(const void *v, int v_dtype, int64_t np, const int64_t *off, int64_t n_cells, int64_t whole,
+                        double *mom, double *m6, cudaStream_t st, int sm_count);
 
-void launch_gather(const void *v, int v_dtype, int64_t np, const int64_t *off, int64_t n_cells, int prec,
-                   double *mom, double *m6, cudaStream_t st) {
+// of n_cells that are a part of a call of `whole` cells
+void launch_gather_part(const void *v, int v_dtype, int64_t np, const int64_t *off, int64_t n_cells, int64_t whole,
+                        int prec, double *mom, double *m6, cudaStream_t st) {
   // FP32 moments of FP32 velocities: shared-memory staged tiles (16-byte
   // aligned velocity arrays); FP32 moments of other arrays: direct loads.
   if (prec != FP_PREC_FP32_MOMENTS)
-    launch_gather_fp64(v, v_dtype, np, off, n_cells, mom, m6, st, sm_count());
+    launch_gather_fp64(v, v_dtype, np, off, n_cells, whole, mom, m6, st, sm_count());
   else if (v_dtype != FP_V_F32 || !launch_gather_tile((const float *)v, np, off, n_cells, mom, m6, st, sm_count()))
     launch_gather_fp32<8>(v, v_dtype, np, off, n_cells, mom, m6, st);
+}
+
+void launch_gather(const void *v, int v_dtype, int64_t np, const int64_t *off, int64_t n_cells, int prec,
+                   double *mom, double *m6, cudaStream_t st) {
+  launch_gather_part(v, v_dtype, np, off, n_cells, n_cells, prec, mom, m6, st);
 }
 
 void launch_solve(const double *mom, const double *tau, int64_t n_cells, const fp_params &p, int prec,

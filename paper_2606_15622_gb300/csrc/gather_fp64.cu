@@ -346,24 +346,27 @@ static void launch_g(const VT *v, int64_t np, const int64_t *off, int64_t n_cell
 }
 
 template <typename VT>
-static void launch_t(const VT *v, int64_t np, const int64_t *off, int64_t n_cells, double *mom, double *m6,
-                     cudaStream_t st, int sm_count) {
+static void launch_t(const VT *v, int64_t np, const int64_t *off, int64_t n_cells, int64_t whole, double *mom,
+                     double *m6, cudaStream_t st, int sm_count) {
   // a whole warp a cell while every cell has a resident warp of its own (the
   // time is one cell's chain then: 400 cells of 100 particles 9.7 us, 14.5
   // with eight lanes); beyond, eight lanes (16: 461 us against 411 on 131,072
-  // cells of 91 particles, 4: 510)
-  if (n_cells <= (int64_t)sm_count * kGBlocksPerSm * kGWarps)
+  // cells of 91 particles, 4: 510).  A part of a larger call takes the whole's
+  // form: the two add in different orders, and a cell's bits do not depend on the
+  // parts that its call is cut into.
+  if (whole <= (int64_t)sm_count * kGBlocksPerSm * kGWarps)
     launch_g<VT, 32>(v, np, off, n_cells, mom, m6, st, sm_count);
   else
     launch_g<VT, 8>(v, np, off, n_cells, mom, m6, st, sm_count);
 }
 
-void launch_gather_fp64(const void *v, int v_dtype, int64_t np, const int64_t *off, int64_t n_cells, double *mom,
-                        double *m6, cudaStream_t st, int sm_count) {
+// whole: the cells of the call that these n_cells are a part of
+void launch_gather_fp64(const void *v, int v_dtype, int64_t np, const int64_t *off, int64_t n_cells, int64_t whole,
+                        double *mom, double *m6, cudaStream_t st, int sm_count) {
   if (v_dtype == FP_V_F32)
-    launch_t<float>((const float *)v, np, off, n_cells, mom, m6, st, sm_count);
+    launch_t<float>((const float *)v, np, off, n_cells, whole, mom, m6, st, sm_count);
   else
-    launch_t<double>((const double *)v, np, off, n_cells, mom, m6, st, sm_count);
+    launch_t<double>((const double *)v, np, off, n_cells, whole, mom, m6, st, sm_count);
 }
 
 }  // namespace fpc

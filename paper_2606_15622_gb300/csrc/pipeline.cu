@@ -27,6 +27,8 @@
 
 namespace fpc {
 int report(int code, const char *msg);
+int moments_of_part(const void *v, int v_dtype, int64_t n_particles, const int64_t *cell_offsets, int64_t n_cells,
+                    int64_t whole, int prec, double *moments_out, double *m6_out, fp_stream_t stream);
 }
 
 struct fp_pipeline {
@@ -168,7 +170,9 @@ int fp_step_host(fp_pipeline *pl, const fp_step_io *io, int v_dtype, int64_t n_p
     cudaStreamWaitEvent(pl->main, pl->ev_h2d[k], 0);
     double *mom = io->d_moments + c0 * FP_NMOM;
     double *m6 = io->d_m6 ? io->d_m6 + c0 : nullptr;
-    if ((rc = fp_moments(io->d_v, v_dtype, n_particles, io->d_offsets + c0, nc, prec, mom, m6, pl->main))) break;
+    if ((rc = fpc::moments_of_part(io->d_v, v_dtype, n_particles, io->d_offsets + c0, nc, n_cells, prec, mom, m6,
+                                   pl->main)))
+      break;
     // ---- the learned closure (moments only) beside the FP64 solve ----
     if (io->net) {
       cudaEventRecord(pl->ev_mom[k], pl->main);
